@@ -74,17 +74,14 @@ constexpr int kSmem =
 // Inverse pass 1 of group-streamed line `lib`: shared memory -> conjugate
 // twiddles -> inverse DFT; emit(lo, x) receives natural-order samples
 // lo + r*S1.
-template <class SC, class Emit>
-__device__ __forceinline__ void b_inverse_pass1(const float2* sm, const float2* tw, int t, Emit&& emit) {
-    constexpr int R1 = SC::R1, S1 = SC::S1, G1 = SC::E / R1;
+template <class SC, int LPB, class Emit>
+__device__ __forceinline__ void b_inverse_pass1(const float2* sm, const float2* tw, int t, int lib, Emit&& emit) {
+    constexpr int R1 = SC::R1, G1 = SC::E / R1;
 #pragma unroll 1
     for (int s = 0; s < G1; ++s) {
-        const int lo = t + SC::T * s;
         float2 x[R1];
-        grp_smem_load<R1, S1>(sm, lo, SC::PADSH, x);
-        grp_twiddle<R1, S1, true>(tw, lo, x);
-        dft_reg<R1, true>(x);
-        emit(lo, x);
+        streamed_final_group<SC, LPB>(sm, tw, t, lib, s, x);
+        emit(t + SC::T * s, x);
     }
 }
 
@@ -102,7 +99,7 @@ __device__ __noinline__ void range_item(const BStrip& st, int line0, int nlines,
         const float2* src = st.raw + (int64_t)(line0 + lib) * SC::N;
         streamed_until_last<SC, G::K, true>(src, sm, st.filt_r, st.tw_r, t, lib);
         // natural-order results back into the slots they were read from
-        b_inverse_pass1<SC>(sm, st.tw_r, t, [&](int lo, const float2 (&x)[R1]) {
+        b_inverse_pass1<SC, G::K>(sm, st.tw_r, t, lib, [&](int lo, const float2 (&x)[R1]) {
 #pragma unroll
             for (int r = 0; r < R1; ++r) sm[smem_pos(lo + r * S1, SC::PADSH)] = x[r];
         });
@@ -129,7 +126,7 @@ __device__ __noinline__ void az_item(const BStrip& st, int line0, int nlines, fl
         float2* row = st.image + (int64_t)(line0 + lib) * st.n_az;
         const int valid = st.n_az;
         streamed_until_last<SC, G::K, true, RAGGED, true>(row, sm, st.filt_a, st.tw_a, t, lib, valid);
-        b_inverse_pass1<SC>(sm, st.tw_a, t, [&](int lo, const float2 (&x)[R1]) {
+        b_inverse_pass1<SC, G::K>(sm, st.tw_a, t, lib, [&](int lo, const float2 (&x)[R1]) {
 #pragma unroll
             for (int r = 0; r < R1; ++r) {
                 const int i = lo + r * S1;

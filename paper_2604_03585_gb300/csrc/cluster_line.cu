@@ -176,41 +176,27 @@ cluster_streamed_kernel(const float2* in, float2* out, int64_t ld, const float2*
     float2* sm = smem_dyn;
     const float2* roots = tw + SC::TW_ELEMS;
     constexpr int R1 = SC::R1, S1 = SC::S1, G1 = SC::E / R1;
-    constexpr int RL = SC::RL, GL = SC::E / RL;
     cluster_first_stage<SC, C, false, false, true>(in + line * ld, G::N, roots, t, rank, sm, cluster);
-    streamed_mid_pass<SC, R1, S1, false, ROLL>(sm, tw, t);
+    streamed_mid_pass<SC, 1, R1, S1, false, ROLL>(sm, tw, t, 0);
     __syncthreads();
     const float2* tw2 = tw + R1 * S1;
     if constexpr (SC::P == 3) {
-        streamed_mid_pass<SC, SC::R2, SC::S2, false, ROLL>(sm, tw2, t);
-        __syncthreads();
+        streamed_mid_pass<SC, 1, SC::R2, SC::S2, false, ROLL, true>(sm, tw2, t, 0);
+        sub_sync<SC, 1>(0);
     }
     // last forward pass, this block's filter slice, first inverse pass
-    const float2* fl = filt + (int64_t)rank * G::M;
-#pragma unroll(ROLL ? 1 : GL)
-    for (int s = 0; s < GL; ++s) {
-        const int g = t + SC::T * s;
-        float2 x[RL];
-        grp_smem_load<RL, 1>(sm, g * RL, SC::PADSH, x);
-        dft_reg<RL, false>(x);
-#pragma unroll
-        for (int r = 0; r < RL; ++r) x[r] = cmul(x[r], fl[(s * RL + r) * SC::T + t]);
-        dft_reg<RL, true>(x);
-        grp_smem_store<RL, 1>(sm, g * RL, SC::PADSH, x);
+    streamed_last_pass<SC, ROLL>(sm, filt + (int64_t)rank * G::M, t);
+    if constexpr (SC::P == 3) {
+        sub_sync<SC, 1>(0);
+        streamed_mid_pass<SC, 1, SC::R2, SC::S2, true, ROLL>(sm, tw2, t, 0);
     }
     __syncthreads();
-    if constexpr (SC::P == 3) {
-        streamed_mid_pass<SC, SC::R2, SC::S2, true, ROLL>(sm, tw2, t);
-        __syncthreads();
-    }
     // inverse pass 1 in place, natural n2 = lo + r S1, times W_N^{-n2 k1}
 #pragma unroll(ROLL ? 1 : G1)
     for (int s = 0; s < G1; ++s) {
         const int lo = t + SC::T * s;
         float2 x[R1];
-        grp_smem_load<R1, S1>(sm, lo, SC::PADSH, x);
-        grp_twiddle<R1, S1, true>(tw, lo, x);
-        dft_reg<R1, true>(x);
+        streamed_final_group<SC, 1>(sm, tw, t, 0, s, x);
 #pragma unroll
         for (int r = 0; r < R1; ++r) x[r] = cmulc(x[r], roots[rank * G::M + lo + r * S1]);
         grp_smem_store<R1, S1>(sm, lo, SC::PADSH, x);
@@ -252,7 +238,7 @@ cluster_dft_kernel(const float2* in, float2* out, int64_t ld, int valid, const f
     for (int s = 0; s < SC::E / SC::RL; ++s) {
 #pragma unroll
         for (int r = 0; r < SC::RL; ++r) {
-            const int k2 = natural_index<SC>(t + SC::T * s, r);
+            const int k2 = natural_index<SC>(pass_group<SC, SC::RL, 1>(t, s), r);
             sm[smem_pos(k2, SC::PADSH)] = v[s * SC::RL + r];
         }
     }

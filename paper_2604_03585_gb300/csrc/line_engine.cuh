@@ -39,6 +39,10 @@ struct Sched {
     static constexpr int PADSH = (RL == 16) ? 4 : (RL == 32) ? 5 : (RL == 64) ? 6 : (RL == 8) ? 3 : (RL == 4) ? 2 : 7;
     static constexpr int SMEM_ELEMS = N + (N >> PADSH);            // per line
     static constexpr int TW_ELEMS = R1 * S1 + ((P == 3) ? R2 * S2 : 0);  // twiddle table length
+    // After pass 1 a line is R1 independent sub-lines of S1 consecutive
+    // positions.  Where a warp's 32 E elements are whole sub-lines, the passes
+    // between the forward and the inverse pass 1 stay inside the warp.
+    static constexpr bool WARP_LOCAL = P == 3 && T % 32 == 0 && (32 * E) % S1 == 0;
     static_assert(R1 * R2 * R3 == N, "radices must multiply to N");
     static_assert(E % R1 == 0 && E % R2 == 0 && E % R3 == 0, "each radix must divide E");
     static_assert((1 << PADSH) == RL, "unsupported last radix");
@@ -48,20 +52,36 @@ struct Sched {
 __device__ __forceinline__ int smem_pos(int p, int padsh) { return p + (p >> padsh); }
 
 // --- pass geometry --------------------------------------------------------
-// Pass with radix R and stride S: thread t's s-th group is g = t + T*s, at
-// positions base(g) + r*S, base(g) = (g / S) * R * S + g % S.
+// Pass with radix R and stride S: group g holds the positions base(g) + r*S,
+// base(g) = (g / S) * R * S + g % S.
 template <int R, int S>
 __device__ __forceinline__ int group_base(int g) { return (g / S) * (R * S) + (g % S); }
 
 template <int R, int S>
 __device__ __forceinline__ int group_lo(int g) { return g % S; }
 
+// Thread t's s-th group of the pass of radix R and stride S.  Pass 1 (S = S1)
+// takes t + T s (coalesced global access).  In the later passes of a
+// WARP_LOCAL schedule warp w takes the 32 E / R consecutive groups of its own
+// sub-lines, so that nothing between the two pass-1 exchanges crosses warps:
+// those exchanges need __syncwarp instead of a barrier of the line, and the
+// warps of a line drift apart, one in its shared-memory phase while another
+// is in its arithmetic (fused pass, 2^24 samples: 67.9 -> 65.8 us at 4096
+// points, 86.4 -> 84.1 at 8192, 112.6 -> 108.8 at 16384).
+template <class SC, int R, int S>
+__device__ __forceinline__ int pass_group(int t, int s) {
+    if constexpr (SC::WARP_LOCAL && S != SC::S1)
+        return (t >> 5) * (32 * (SC::E / R)) + 32 * s + (t & 31);
+    else
+        return t + SC::T * s;
+}
+
 // --- shared-memory exchange ----------------------------------------------
 template <class SC, int R, int S>
 __device__ __forceinline__ void smem_store(float2* sm, int t, const float2 (&v)[SC::E]) {
 #pragma unroll
     for (int s = 0; s < SC::E / R; ++s) {
-        const int base = group_base<R, S>(t + SC::T * s);
+        const int base = group_base<R, S>(pass_group<SC, R, S>(t, s));
 #pragma unroll
         for (int r = 0; r < R; ++r) sm[smem_pos(base + r * S, SC::PADSH)] = v[s * R + r];
     }
@@ -70,7 +90,7 @@ template <class SC, int R, int S>
 __device__ __forceinline__ void smem_load(const float2* sm, int t, float2 (&v)[SC::E]) {
 #pragma unroll
     for (int s = 0; s < SC::E / R; ++s) {
-        const int base = group_base<R, S>(t + SC::T * s);
+        const int base = group_base<R, S>(pass_group<SC, R, S>(t, s));
 #pragma unroll
         for (int r = 0; r < R; ++r) v[s * R + r] = sm[smem_pos(base + r * S, SC::PADSH)];
     }
@@ -96,7 +116,7 @@ template <class SC, int R, int S, bool INV>
 __device__ __forceinline__ void twiddle_groups(const float2* tw, int t, float2 (&v)[SC::E]) {
 #pragma unroll
     for (int s = 0; s < SC::E / R; ++s) {
-        const int lo = group_lo<R, S>(t + SC::T * s);
+        const int lo = group_lo<R, S>(pass_group<SC, R, S>(t, s));
 #pragma unroll
         for (int r = 1; r < R; ++r) {
             const float2 w = tw[r * S + lo];
@@ -136,11 +156,23 @@ __device__ __forceinline__ void global_store(float2* dst, int valid, int t, cons
 
 // --- the matched-filter multiply in last-pass geometry --------------------
 // filt[(s*RL + r)*T + t] = H[k(P)] / N for the element at position
-// P = g*RL + r, g = t + T*s; coalesced for fixed (s, r).
+// P = g*RL + r, g = t + T*s; coalesced for fixed (s, r).  filter_row: the
+// slot of r = 0 of thread t's s-th group; slot r is r*T further.
+template <class SC>
+__device__ __forceinline__ int filter_row(int t, int s) {
+    if constexpr (!SC::WARP_LOCAL) return s * (SC::RL * SC::T) + t;
+    const int g = pass_group<SC, SC::RL, 1>(t, s);
+    return g / SC::T * (SC::RL * SC::T) + g % SC::T;
+}
+
 template <class SC>
 __device__ __forceinline__ void filter_multiply(const float2* filt, int t, float2 (&v)[SC::E]) {
 #pragma unroll
-    for (int j = 0; j < SC::E; ++j) v[j] = cmul(v[j], filt[j * SC::T + t]);
+    for (int s = 0; s < SC::E / SC::RL; ++s) {
+        const float2* f = filt + filter_row<SC>(t, s);
+#pragma unroll
+        for (int r = 0; r < SC::RL; ++r) v[s * SC::RL + r] = cmul(v[s * SC::RL + r], f[r * SC::T]);
+    }
 }
 
 // --- line synchronisation among the T threads of one line ----------------
@@ -159,6 +191,49 @@ __device__ __forceinline__ void line_sync(int line_in_block) {
     }
 }
 
+// --- synchronisation of an exchange between two passes after pass 1 --------
+template <class SC, int LPB>
+__device__ __forceinline__ void sub_sync(int line_in_block) {
+    if constexpr (SC::WARP_LOCAL)
+        __syncwarp();
+    else
+        line_sync<SC, LPB>(line_in_block);
+}
+
+// --- staggered starts after a barrier of the line ---------------------------
+// Released together by a barrier, all warps of a line load from shared memory
+// at once, then compute at once, and the two units take turns idling (16384
+// points, one block per SM: L1 41 %, FMA 40 %, issue 42 % busy).  With lines
+// of at least eight warps, warps start in four groups, each once the one
+// before has issued its loads (a named barrier that the group before arrives
+// at and does not wait for), which keeps them out of phase: 84.1 -> 78.3 us at
+// 8192, 108.8 -> 102.6 at 16384 (2^24 samples).  Blocks of four warps gain
+// nothing (four to five blocks per SM are out of phase already; 65.8 -> 67.7
+// at 4096).  Barrier ids 9 ... 15 (8 + 4 line + 1 ... 3), so for one or two
+// lines per block; the lines of a block synchronise on ids 0 ... 8.
+template <class SC, int LPB>
+struct Stagger {
+    static constexpr bool ON = SC::WARP_LOCAL && SC::T >= 256 && LPB <= 2;
+    static constexpr int GROUP = ON ? SC::T / 4 : SC::T;
+};
+template <class SC, int LPB>
+__device__ __forceinline__ void stagger_wait(int t, int line_in_block) {
+    if constexpr (Stagger<SC, LPB>::ON) {
+        constexpr int GROUP = Stagger<SC, LPB>::GROUP;
+        const int k = t / GROUP;
+        if (k > 0) asm volatile("bar.sync %0, %1;" ::"r"(8 + 4 * line_in_block + k), "r"(2 * GROUP) : "memory");
+    }
+}
+template <class SC, int LPB>
+__device__ __forceinline__ void stagger_release(int t, int line_in_block) {
+    if constexpr (Stagger<SC, LPB>::ON) {
+        constexpr int GROUP = Stagger<SC, LPB>::GROUP;
+        const int k = t / GROUP;
+        if (k < 3)
+            asm volatile("bar.arrive %0, %1;" ::"r"(8 + 4 * line_in_block + k + 1), "r"(2 * GROUP) : "memory");
+    }
+}
+
 // --- forward transform (all passes), leaving the digit-reversed spectrum
 //     in registers in last-pass geometry ---------------------------------
 template <class SC, int LPB>
@@ -173,7 +248,7 @@ __device__ __forceinline__ void forward_passes(float2 (&v)[SC::E], float2* sm, c
     if constexpr (SC::P == 3) {
         twiddle_groups<SC, SC::R2, SC::S2, false>(tw + SC::R1 * SC::S1, t, v);
         smem_store<SC, SC::R2, SC::S2>(sm, t, v);
-        line_sync<SC, LPB>(lib);
+        sub_sync<SC, LPB>(lib);
         smem_load<SC, SC::R3, SC::S3>(sm, t, v);
         dft_groups<SC, SC::R3, false>(v);
     }
@@ -187,7 +262,7 @@ __device__ __forceinline__ void inverse_passes(float2 (&v)[SC::E], float2* sm, c
     if constexpr (SC::P == 3) {
         dft_groups<SC, SC::R3, true>(v);
         smem_store<SC, SC::R3, SC::S3>(sm, t, v);
-        line_sync<SC, LPB>(lib);
+        sub_sync<SC, LPB>(lib);
         smem_load<SC, SC::R2, SC::S2>(sm, t, v);
         twiddle_groups<SC, SC::R2, SC::S2, true>(tw + SC::R1 * SC::S1, t, v);
     }
@@ -202,6 +277,17 @@ __device__ __forceinline__ void inverse_passes(float2 (&v)[SC::E], float2* sm, c
 // ---------------------------------------------------------------------------
 // Kernels
 // ---------------------------------------------------------------------------
+// Blocks per SM at 128 registers a thread, sixteen warps, for the three-pass
+// E = 32 engines.  The compiler's own choice falls on either side of it: 96
+// registers and a fifth block, whose shared memory takes the place of the
+// twiddle and filter tables in L1 (fused pass at 4096 points, 2^24 samples:
+// 69.8 us against 65.8), or above 128 and one block less (plain transform of
+// 8192 points: 141 registers, one block, 85.7 us against 65.7).
+template <class SC, int LPB>
+__host__ __device__ constexpr int min_blocks_128() {
+    return SC::P == 3 && SC::E == 32 && SC::T * LPB <= 512 ? 512 / (SC::T * LPB) : 0;
+}
+
 // Every kernel takes n_lines lines of length N; line l starts at
 // data + l*ld and holds `valid` (<= N) stored samples: samples beyond `valid`
 // are read as zeros and never written (zero-padded transforms).
@@ -258,7 +344,7 @@ __device__ __forceinline__ int natural_index(int g, int r) {
 }
 
 template <class SC, int LPB, bool INV>
-__global__ void __launch_bounds__(SC::T * LPB)
+__global__ void __launch_bounds__(SC::T * LPB, min_blocks_128<SC, LPB>())
 dft_lines_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld,
                  int valid, const float2* tw) {
     extern __shared__ float2 smem_dyn[];
@@ -283,7 +369,7 @@ dft_lines_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld,
     for (int s = 0; s < SC::E / SC::RL; ++s) {
 #pragma unroll
         for (int r = 0; r < SC::RL; ++r) {
-            const int k = natural_index<SC>(t + SC::T * s, r);
+            const int k = natural_index<SC>(pass_group<SC, SC::RL, 1>(t, s), r);
             sm[smem_pos(k, SC::PADSH)] = v[s * SC::RL + r];
         }
     }

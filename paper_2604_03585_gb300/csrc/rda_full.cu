@@ -194,7 +194,7 @@ rcmc_tile_kernel(const float2* __restrict__ in, float2* __restrict__ out, int n_
 // conj(FFT(conj .)) (Sec. II-C).  Otherwise the forward FFT of the line (the
 // Range-Doppler domain, Sec. IV-A step 2).
 template <class SC, bool COMPRESS>
-__global__ void __launch_bounds__(SC::T)
+__global__ void __launch_bounds__(SC::T, min_blocks_128<SC, 1>())
 az_streamed_kernel(const float2* in, float2* out, int64_t n_lines, const float2* tw, const RdColumn* cols,
                    double r_near) {
     extern __shared__ float2 smem_dyn[];
@@ -245,15 +245,15 @@ az_streamed_kernel(const float2* in, float2* out, int64_t n_lines, const float2*
     }
     __syncthreads();
     if constexpr (SC::P == 3) {
-        streamed_mid_pass<SC, SC::R2, SC::S2, false, true>(sm, tw + R1 * S1, t);
-        __syncthreads();
+        streamed_mid_pass<SC, 1, SC::R2, SC::S2, false, true, true>(sm, tw + R1 * S1, t, 0);
+        sub_sync<SC, 1>(0);
     }
     // last pass into registers, then natural order through shared memory
     float2 v[SC::E];
 #pragma unroll
     for (int s = 0; s < GL; ++s) {
         float2 x[RL];
-        grp_smem_load<RL, 1>(sm, (t + SC::T * s) * RL, SC::PADSH, x);
+        grp_smem_load<RL, 1>(sm, pass_group<SC, RL, 1>(t, s) * RL, SC::PADSH, x);
         dft_reg<RL, false>(x);
 #pragma unroll
         for (int r = 0; r < RL; ++r) v[s * RL + r] = x[r];
@@ -262,7 +262,7 @@ az_streamed_kernel(const float2* in, float2* out, int64_t n_lines, const float2*
 #pragma unroll
     for (int s = 0; s < GL; ++s) {
 #pragma unroll
-        for (int r = 0; r < RL; ++r) sm[smem_pos(natural_index<SC>(t + SC::T * s, r), SC::PADSH)] = v[s * RL + r];
+        for (int r = 0; r < RL; ++r) sm[smem_pos(natural_index<SC>(pass_group<SC, RL, 1>(t, s), r), SC::PADSH)] = v[s * RL + r];
     }
     __syncthreads();
     constexpr float inv_n = 1.0f / SC::N;

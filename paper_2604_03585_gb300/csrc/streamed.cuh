@@ -40,15 +40,18 @@ __device__ __forceinline__ void grp_twiddle(const float2* tw, int lo, float2 (&g
 
 // One middle pass (shared memory in, shared memory out) of radix R, stride S.
 // FWD: DFT then twiddle; inverse: conjugate twiddle then inverse DFT.
-template <class SC, int R, int S, bool INV, bool ROLL>
-__device__ __forceinline__ void streamed_mid_pass(float2* sm, const float2* tw, int t) {
+// STAGGER: the pass follows a barrier of the whole line.
+template <class SC, int LPB, int R, int S, bool INV, bool ROLL, bool STAGGER = false>
+__device__ __forceinline__ void streamed_mid_pass(float2* sm, const float2* tw, int t, int lib) {
     constexpr int G = SC::E / R;
 #pragma unroll(ROLL ? 1 : G)
     for (int s = 0; s < G; ++s) {
-        const int g = t + SC::T * s;
+        const int g = pass_group<SC, R, S>(t, s);
         const int base = group_base<R, S>(g);
         float2 x[R];
+        if (STAGGER && s == 0) stagger_wait<SC, LPB>(t, lib);
         grp_smem_load<R, S>(sm, base, SC::PADSH, x);
+        if (STAGGER && s == 0) stagger_release<SC, LPB>(t, lib);
         if (!INV) {
             dft_reg<R, false>(x);
             grp_twiddle<R, S, false>(tw, group_lo<R, S>(g), x);
@@ -57,6 +60,25 @@ __device__ __forceinline__ void streamed_mid_pass(float2* sm, const float2* tw, 
             dft_reg<R, true>(x);
         }
         grp_smem_store<R, S>(sm, base, SC::PADSH, x);
+    }
+}
+
+// The last forward pass, the filter multiply and the first inverse pass, one
+// group at a time.
+template <class SC, bool ROLL>
+__device__ __forceinline__ void streamed_last_pass(float2* sm, const float2* filt, int t) {
+    constexpr int RL = SC::RL, GL = SC::E / RL;
+#pragma unroll(ROLL ? 1 : GL)
+    for (int s = 0; s < GL; ++s) {
+        const int g = pass_group<SC, RL, 1>(t, s);
+        const float2* f = filt + filter_row<SC>(t, s);
+        float2 x[RL];
+        grp_smem_load<RL, 1>(sm, g * RL, SC::PADSH, x);
+        dft_reg<RL, false>(x);
+#pragma unroll
+        for (int r = 0; r < RL; ++r) x[r] = cmul(x[r], f[r * SC::T]);
+        dft_reg<RL, true>(x);
+        grp_smem_store<RL, 1>(sm, g * RL, SC::PADSH, x);
     }
 }
 
@@ -85,7 +107,6 @@ template <class SC, int LPB, bool ROLL, bool RAGGED = false, bool L2ONLY = false
 __device__ __forceinline__ void streamed_until_last(const float2* src, float2* sm, const float2* filt,
                                                     const float2* tw, int t, int lib, int valid = SC::N) {
     constexpr int R1 = SC::R1, S1 = SC::S1, G1 = SC::E / R1;
-    constexpr int RL = SC::RL, GL = SC::E / RL;
 
     // ---- forward pass 1: HBM -> DFT -> twiddle -> shared memory, with the
     //      next group's loads in flight during the current group's arithmetic
@@ -111,26 +132,28 @@ __device__ __forceinline__ void streamed_until_last(const float2* src, float2* s
     line_sync<SC, LPB>(lib);
     const float2* tw2 = tw + SC::R1 * SC::S1;
     if constexpr (SC::P == 3) {
-        streamed_mid_pass<SC, SC::R2, SC::S2, false, ROLL>(sm, tw2, t);
-        line_sync<SC, LPB>(lib);
+        streamed_mid_pass<SC, LPB, SC::R2, SC::S2, false, ROLL, true>(sm, tw2, t, lib);
+        sub_sync<SC, LPB>(lib);
     }
-    // ---- last forward pass, filter, first inverse pass: one group at a time
-#pragma unroll(ROLL ? 1 : GL)
-    for (int s = 0; s < GL; ++s) {
-        const int g = t + SC::T * s;
-        float2 x[RL];
-        grp_smem_load<RL, 1>(sm, g * RL, SC::PADSH, x);
-        dft_reg<RL, false>(x);
-#pragma unroll
-        for (int r = 0; r < RL; ++r) x[r] = cmul(x[r], filt[(s * RL + r) * SC::T + t]);
-        dft_reg<RL, true>(x);
-        grp_smem_store<RL, 1>(sm, g * RL, SC::PADSH, x);
+    streamed_last_pass<SC, ROLL>(sm, filt, t);
+    if constexpr (SC::P == 3) {
+        sub_sync<SC, LPB>(lib);
+        streamed_mid_pass<SC, LPB, SC::R2, SC::S2, true, ROLL>(sm, tw2, t, lib);
     }
     line_sync<SC, LPB>(lib);
-    if constexpr (SC::P == 3) {
-        streamed_mid_pass<SC, SC::R2, SC::S2, true, ROLL>(sm, tw2, t);
-        line_sync<SC, LPB>(lib);
-    }
+}
+
+// One group of the inverse pass 1 of a line left by streamed_until_last: the
+// natural-order samples lo + r*S1 (lo = t + T s) in x.
+template <class SC, int LPB>
+__device__ __forceinline__ void streamed_final_group(const float2* sm, const float2* tw, int t, int lib, int s,
+                                                     float2 (&x)[SC::R1]) {
+    const int lo = t + SC::T * s;
+    if (s == 0) stagger_wait<SC, LPB>(t, lib);
+    grp_smem_load<SC::R1, SC::S1>(sm, lo, SC::PADSH, x);
+    if (s == 0) stagger_release<SC, LPB>(t, lib);
+    grp_twiddle<SC::R1, SC::S1, true>(tw, lo, x);
+    dft_reg<SC::R1, true>(x);
 }
 
 template <class SC, int LPB, bool ROLL>
@@ -150,9 +173,7 @@ __device__ __forceinline__ void fused_streamed_body(const float2* in, float2* ou
     for (int s = 0; s < G1; ++s) {
         const int lo = t + SC::T * s;
         float2 x[R1];
-        grp_smem_load<R1, S1>(sm, lo, SC::PADSH, x);
-        grp_twiddle<R1, S1, true>(tw, lo, x);
-        dft_reg<R1, true>(x);
+        streamed_final_group<SC, LPB>(sm, tw, t, lib, s, x);
 #pragma unroll
         for (int r = 0; r < R1; ++r) __stcs(dst + lo + r * S1, x[r]);
     }
@@ -180,7 +201,7 @@ __device__ __forceinline__ int find_seg(const int64_t* line_begin, int n_seg, in
 }
 
 template <class SC, int LPB, bool ROLL, bool RAGGED>
-__global__ void __launch_bounds__(SC::T * LPB)
+__global__ void __launch_bounds__(SC::T * LPB, min_blocks_128<SC, LPB>())
 fused_seg_kernel(const Seg* segs, const int64_t* line_begin, int n_seg, int64_t n_lines, const float2* filt,
                  const float2* tw) {
     extern __shared__ float2 smem_dyn[];
@@ -199,9 +220,7 @@ fused_seg_kernel(const Seg* segs, const int64_t* line_begin, int n_seg, int64_t 
     for (int s = 0; s < G1; ++s) {
         const int lo = t + SC::T * s;
         float2 x[R1];
-        grp_smem_load<R1, S1>(sm, lo, SC::PADSH, x);
-        grp_twiddle<R1, S1, true>(tw, lo, x);
-        dft_reg<R1, true>(x);
+        streamed_final_group<SC, LPB>(sm, tw, t, lib, s, x);
 #pragma unroll
         for (int r = 0; r < R1; ++r) {
             const int i = lo + r * S1;
@@ -233,11 +252,8 @@ __device__ __forceinline__ void fused_range_ct_body(const float2* in, float2* im
     float2 v[SC::E];
 #pragma unroll
     for (int s = 0; s < G1; ++s) {
-        const int lo = t + SC::T * s;
         float2 x[R1];
-        grp_smem_load<R1, S1>(sm, lo, SC::PADSH, x);
-        grp_twiddle<R1, S1, true>(tw, lo, x);
-        dft_reg<R1, true>(x);
+        streamed_final_group<SC, QL>(sm, tw, t, lib, s, x);
 #pragma unroll
         for (int r = 0; r < R1; ++r) v[s * R1 + r] = x[r];
     }
@@ -316,11 +332,8 @@ __device__ __forceinline__ void fused_range_ct_cluster_body(const float2* in, fl
     float2 v[SC::E];
 #pragma unroll
     for (int s = 0; s < G1; ++s) {
-        const int lo = t + SC::T * s;
         float2 x[R1];
-        grp_smem_load<R1, S1>(sm, lo, SC::PADSH, x);
-        grp_twiddle<R1, S1, true>(tw, lo, x);
-        dft_reg<R1, true>(x);
+        streamed_final_group<SC, 1>(sm, tw, t, 0, s, x);
 #pragma unroll
         for (int r = 0; r < R1; ++r) v[s * R1 + r] = x[r];
     }
@@ -415,7 +428,7 @@ fused_range_ct_kernel(const float2* in, float2* img, int64_t n_lines, int64_t ld
 }
 
 template <class SC, int LPB, bool ROLL>
-__global__ void __launch_bounds__(SC::T * LPB)
+__global__ void __launch_bounds__(SC::T * LPB, min_blocks_128<SC, LPB>())
 fused_streamed_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, const float2* filt,
                       const float2* tw) {
     fused_streamed_body<SC, LPB, ROLL>(in, out, n_lines, ld, filt, tw);

@@ -21,7 +21,7 @@
 namespace sar {
 
 template <class SC, int LPB, bool ROLL>
-__global__ void __launch_bounds__(SC::T * LPB)
+__global__ void __launch_bounds__(SC::T * LPB, min_blocks_128<SC, LPB>())
 fused_wrap_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, int n, const float2* filt,
                   const float2* tw) {
     extern __shared__ float2 smem_dyn[];
@@ -37,9 +37,7 @@ fused_wrap_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, in
     for (int s = 0; s < G1; ++s) {
         const int lo = t + SC::T * s;
         float2 x[R1];
-        grp_smem_load<R1, S1>(sm, lo, SC::PADSH, x);
-        grp_twiddle<R1, S1, true>(tw, lo, x);
-        dft_reg<R1, true>(x);
+        streamed_final_group<SC, LPB>(sm, tw, t, lib, s, x);
         grp_smem_store<R1, S1>(sm, lo, SC::PADSH, x);
     }
     line_sync<SC, LPB>(lib);
@@ -62,7 +60,7 @@ fused_wrap_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, in
 // inverse pass leaves the convolution there, and the store applies c_k.  INV:
 // the inverse kernel as conj(DFT(conj x)).  chirp[m] = c_m, m < n.
 template <class SC, int LPB, bool ROLL, bool INV>
-__global__ void __launch_bounds__(SC::T * LPB)
+__global__ void __launch_bounds__(SC::T * LPB, min_blocks_128<SC, LPB>())
 bluestein_dft_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, int n, const float2* filt,
                      const float2* tw, const float2* chirp) {
     extern __shared__ float2 smem_dyn[];
@@ -83,36 +81,24 @@ bluestein_dft_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld,
         sm[smem_pos(j, SC::PADSH)] = a;
     }
     line_sync<SC, LPB>(lib);
-    streamed_mid_pass<SC, R1, S1, false, ROLL>(sm, tw, t);
+    streamed_mid_pass<SC, LPB, R1, S1, false, ROLL>(sm, tw, t, lib);
     line_sync<SC, LPB>(lib);
     const float2* tw2 = tw + R1 * S1;
     if constexpr (SC::P == 3) {
-        streamed_mid_pass<SC, SC::R2, SC::S2, false, ROLL>(sm, tw2, t);
-        line_sync<SC, LPB>(lib);
+        streamed_mid_pass<SC, LPB, SC::R2, SC::S2, false, ROLL, true>(sm, tw2, t, lib);
+        sub_sync<SC, LPB>(lib);
     }
-#pragma unroll(ROLL ? 1 : GL)
-    for (int s = 0; s < GL; ++s) {
-        const int g = t + SC::T * s;
-        float2 x[RL];
-        grp_smem_load<RL, 1>(sm, g * RL, SC::PADSH, x);
-        dft_reg<RL, false>(x);
-#pragma unroll
-        for (int r = 0; r < RL; ++r) x[r] = cmul(x[r], filt[(s * RL + r) * SC::T + t]);
-        dft_reg<RL, true>(x);
-        grp_smem_store<RL, 1>(sm, g * RL, SC::PADSH, x);
+    streamed_last_pass<SC, ROLL>(sm, filt, t);
+    if constexpr (SC::P == 3) {
+        sub_sync<SC, LPB>(lib);
+        streamed_mid_pass<SC, LPB, SC::R2, SC::S2, true, ROLL>(sm, tw2, t, lib);
     }
     line_sync<SC, LPB>(lib);
-    if constexpr (SC::P == 3) {
-        streamed_mid_pass<SC, SC::R2, SC::S2, true, ROLL>(sm, tw2, t);
-        line_sync<SC, LPB>(lib);
-    }
 #pragma unroll(ROLL ? 1 : G1)
     for (int s = 0; s < G1; ++s) {
         const int lo = t + SC::T * s;
         float2 x[R1];
-        grp_smem_load<R1, S1>(sm, lo, SC::PADSH, x);
-        grp_twiddle<R1, S1, true>(tw, lo, x);
-        dft_reg<R1, true>(x);
+        streamed_final_group<SC, LPB>(sm, tw, t, lib, s, x);
         grp_smem_store<R1, S1>(sm, lo, SC::PADSH, x);
     }
     line_sync<SC, LPB>(lib);
