@@ -346,7 +346,7 @@ typedef struct sar_batch_s *sar_batch;
 typedef struct {
     int64_t strips;          /* strips in the batch */
     int64_t samples;         /* sum of n_az * n_range */
-    int64_t work_bytes;      /* batch-owned scratch (range-compressed strips) */
+    int64_t work_bytes;      /* batch-owned scratch (range-compressed strips, or the one-launch kernel's) */
     int32_t kernels_per_run; /* kernels in the graph */
     int32_t range_classes;   /* distinct (n_range, range spectrum) */
     int32_t azimuth_classes; /* distinct (L, azimuth spectrum) */
@@ -357,14 +357,16 @@ typedef struct {
  * azimuth spectrum)), build each class's filter and twiddle tables, and
  * capture the whole batch into one CUDA graph.
  * flags 0: the graph is one memset and ONE persistent kernel.  Each resident
- * block (one per SM) takes work items from one list: range items (k azimuth
- * rows of a strip, k = 16384 / n_range, compressed along range and written
- * straight into the corner-turned image, Sec. IV-A steps 1-2) and azimuth
- * items (k range bins, compressed along azimuth in place, Sec. IV-A step 4).
+ * block (one per SM) takes work items: first range items (at least four
+ * azimuth rows of a strip, compressed along range and written straight into
+ * the corner-turned image, Sec. IV-A steps 1-2), then each quarter of the
+ * block azimuth items (range bins, compressed along azimuth in place, Sec.
+ * IV-A step 4; above 4096 samples the whole block).
  * A strip's azimuth items wait on a device counter of its finished range
  * lines; that wait is bounded (about a second of SM clock, SAR_WAIT_CYCLES),
  * and a run whose wait ran out is reported by sar_batch_status.  No work
- * buffer.
+ * buffer, but for strips of 8192 or 16384 range samples a scratch of up to
+ * 384 KiB per SM (without memory for it those strips run slower).
  * flags SAR_BATCH_MULTI_KERNEL or SAR_BATCH_EXACT_AZIMUTH: see below (one
  * launch per class, a batched corner turn, a work buffer of 8 bytes per raw
  * sample).

@@ -5,7 +5,7 @@
 // count); its azimuth lines are transformed at L = max(256, next power of
 // two >= n_az), zero-padded, and the image keeps its n_az columns.
 //
-// Default: one persistent kernel (batch_persistent.cu) walks a list of work
+// Default: one persistent kernel (batch_persistent.cu) walks two lists of work
 // items -- range items (k azimuth rows of a strip, compressed along range and
 // written corner-turned into the image) and azimuth items (k range bins,
 // compressed in place) -- with per-strip completion counters between a
@@ -143,7 +143,8 @@ struct sar_batch_s {
     sar::TSeg *tsegs_dev = nullptr;
     int64_t *tbegin_dev = nullptr;
     void *tables = nullptr;    // filters, twiddles, segment tables
-    void *work = nullptr;      // range-compressed strips
+    void *work = nullptr;      // range-compressed strips; one-launch path: scratch of its long range items
+    int64_t work_bytes = 0;    // of that scratch
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int device = 0;
@@ -196,7 +197,7 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, sar_
     auto class_of = [&](int64_t n, const void *spec, bool range) -> int {
         for (size_t i = 0; i < cls.size(); ++i)
             if (cls[i].n == n && cls[i].spectrum == spec && cls[i].range == range) return (int)i;
-        const char *name = sar::batch_schedule_name((int)n);
+        const char *name = sar::batch_geometry((int)n).schedule;
         const SchedDesc *d = name ? sar::find_schedule(name) : nullptr;
         if (!d) return -1;
         cls.push_back(TClass{d, spec, n, range});
@@ -215,31 +216,91 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, sar_
         ac[i] = class_of(L[i], strips[i].az_spectrum, false);
         if (rc[i] < 0 || ac[i] < 0) return sar::report_error(SAR_ERR_UNSUPPORTED, "no batch engine for a strip length");
     }
-    // item list: strips largest first; range items of strip j + 1 before the
-    // azimuth items of strip j, so that an azimuth item's strip is finished
-    // (or being finished by blocks that took its items earlier) when a block
-    // takes it
+    if (const cudaError_t pe = sar::prepare_batch_persistent(); pe != cudaSuccess || sar::batch_grid() <= 0) {
+        cudaGetLastError();
+        return sar::report_error(SAR_ERR_CUDA, "the batch kernel does not fit the device");
+    }
+    // how the range items of each length run.  Long lines are stored in sets of
+    // four, all but the last parked in the scratch (none if there is no memory
+    // for it: then an item is the lines its worker holds at once).  Where that
+    // would leave workers idle, the whole block takes as many lines as it holds
+    // and parks none: below two sets for each worker of 128 threads at 2048 and
+    // 4096 samples (one strip of 4096 x 400: 37 us against 90), below one set
+    // for each block at 8192 (8192 x 300: 53 us against 108; x 1000: 178
+    // against 157) and 16384 (x 300: 110 against 137; x 1000: 352 against 307)
+    const int64_t blocks = sar::batch_grid(), workers = blocks * (sar::kBatchThreads / 128);
+    int64_t sets_short = 0, sets_8192 = 0, sets_16384 = 0, sets_tiny = 0;
+    for (int32_t i = 0; i < count; ++i) {
+        const int64_t sets = (strips[i].n_az + sar::kLongLines - 1) / sar::kLongLines;
+        if (strips[i].n_range == 16384) sets_16384 += sets;
+        else if (strips[i].n_range == 8192) sets_8192 += sets;
+        else if (strips[i].n_range >= 2048) sets_short += sets;
+        else if (strips[i].n_range <= 512) sets_tiny += (strips[i].n_az + 7) / 8;
+    }
+    auto few = [&](int64_t n) {
+        return n == 16384 ? sets_16384 < blocks : n == 8192 ? sets_8192 < blocks : sets_short < 2 * workers;
+    };
+    auto range_geometry = [&](int64_t n) {
+        sar::BatchGeom g = sar::batch_geometry((int)n, few(n));
+        if (n >= 8192 && few(n)) g.parks = false, g.set = g.lines;
+        return g;
+    };
+    bool parks = false;
+    for (int32_t i = 0; i < count; ++i) parks = parks || range_geometry(strips[i].n_range).parks;
+    if (parks) {
+        const size_t bytes = sizeof(float2) * (size_t)sar::batch_grid() * sar::kBatchScratch;
+        if (cudaMalloc(&b->work, bytes) == cudaSuccess) {
+            b->work_bytes = (int64_t)bytes;
+        } else {
+            cudaGetLastError();
+            b->work = nullptr;
+        }
+    }
+    // item lists, strips of long range lines first (their items take longest),
+    // then the largest.  A range item is one set, so that neighbouring sets,
+    // whose 32-byte runs share the image rows' L2 lines, are stored at about
+    // the same time (1024 x 3651 strips: 228 us per 2^24 samples against 271
+    // with four sets per item), or up to 8192 samples of lines up to 512, where
+    // taking the item would cost more (256 x 4096: 176 against 204); an azimuth item of 128 threads is up to four rounds of its worker's
+    // lines where that leaves every worker several (256 x 4096: 176 against
+    // 208 with one)
     std::vector<int32_t> order(count);
     for (int32_t i = 0; i < count; ++i) order[i] = i;
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
-        return strips[x].n_az * strips[x].n_range > strips[y].n_az * strips[y].n_range;
+        if (strips[x].n_range != strips[y].n_range) return strips[x].n_range > strips[y].n_range;
+        return strips[x].n_az > strips[y].n_az;
     });
     std::vector<sar::BItem> items;
-    auto add_range = [&](int32_t i) {
-        const int k = sar::batch_lines_per_item((int)strips[i].n_range);
-        for (int64_t a = 0; a < strips[i].n_az; a += k)
-            items.push_back(sar::BItem{0, i, (int32_t)a, (int32_t)std::min<int64_t>(k, strips[i].n_az - a)});
+    sar::BatchLists lists = {};
+    auto add_list = [&](int list, bool range, int threads) {
+        int per_item = 1;   // rounds or sets
+        if (!range && threads == 128) {
+            int64_t rounds = 0;
+            for (int32_t i : order) {
+                const sar::BatchGeom g = sar::batch_geometry((int)L[i]);
+                if (g.threads == threads) rounds += (strips[i].n_range + g.lines - 1) / g.lines;
+            }
+            per_item = (int)std::max<int64_t>(1, std::min<int64_t>(4, rounds / (4 * workers)));
+        }
+        for (int32_t i : order) {
+            const sar::BatchGeom g =
+                range ? range_geometry(strips[i].n_range) : sar::batch_geometry((int)L[i]);
+            if (g.threads != threads) continue;
+            const int64_t lines = range ? strips[i].n_az : strips[i].n_range, n = range ? strips[i].n_range : L[i];
+            const int unit = range && (b->work || !g.parks) ? g.set : g.lines;
+            const int64_t tiny = std::min<int64_t>(8192 / (unit * n), sets_tiny / (2 * workers));
+            const int k = unit * (range && n <= 512 ? (int)std::max<int64_t>(1, tiny) : per_item);
+            for (int64_t l = 0; l < lines; l += k)
+                items.push_back(sar::BItem{range ? 0 : 1, i, (int32_t)l, (int32_t)std::min<int64_t>(k, lines - l)});
+        }
+        lists.begin[list + 1] = (int32_t)items.size();
     };
-    auto add_az = [&](int32_t i) {
-        const int k = sar::batch_lines_per_item((int)L[i]);
-        for (int64_t r = 0; r < strips[i].n_range; r += k)
-            items.push_back(sar::BItem{1, i, (int32_t)r, (int32_t)std::min<int64_t>(k, strips[i].n_range - r)});
-    };
-    for (int32_t j = 0; j < count; ++j) {
-        add_range(order[j]);
-        if (j > 0) add_az(order[j - 1]);
-    }
-    add_az(order[count - 1]);
+    add_list(0, true, 512);
+    add_list(1, true, 256);
+    add_list(2, true, 128);
+    add_list(2, false, 128);
+    add_list(3, false, 256);
+    add_list(4, false, 512);
     if (items.size() > (size_t)0x7fffffff) return sar::report_error(SAR_ERR_UNSUPPORTED, "too many work items");
 
     // ---- device memory: tables, strips, items, counters, status
@@ -258,7 +319,7 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, sar_
     }
     const size_t off_st = reserve(sizeof(sar::BStrip) * count);
     const size_t off_it = reserve(sizeof(sar::BItem) * items.size());
-    const size_t off_ctr = reserve(sizeof(int) * ((size_t)count + 1));
+    const size_t off_ctr = reserve(sizeof(int) * ((size_t)count + sar::kBatchNumLists));
     const size_t off_status = reserve(sizeof(int));
     const size_t off_ix = reserve(sizeof(int32_t) * max_n);
     if (cudaMalloc(&b->tables, tab) != cudaSuccess) {
@@ -275,7 +336,6 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, sar_
     cudaStream_t s = nullptr;
     cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();   // the caller's spectra are ready
-    if (e == cudaSuccess) e = sar::prepare_batch_persistent();
     std::vector<int32_t> idx;
     for (size_t ci = 0; ci < cls.size() && e == cudaSuccess; ++ci) {
         TClass &c = cls[ci];
@@ -305,13 +365,19 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, sar_
         e = cudaMemcpyAsync(items_dev, items.data(), sizeof(sar::BItem) * items.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->status_dev, 0, sizeof(int), s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    lists.items = items_dev;
+    lists.strips = strips_dev;
+    lists.done = counters;
+    lists.next = counters + count;
+    lists.status = b->status_dev;
+    lists.wait_cycles = batch_wait_cycles();
+    lists.scratch = (float2 *)b->work;
     // ---- the graph: clear the counters, one kernel
     if (e == cudaSuccess) e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t le = cudaMemsetAsync(counters, 0, sizeof(int) * ((size_t)count + 1), s);
+        cudaError_t le = cudaMemsetAsync(counters, 0, sizeof(int) * ((size_t)count + sar::kBatchNumLists), s);
         if (le == cudaSuccess)
-            le = sar::launch_batch_persistent(items_dev, (int)items.size(), strips_dev, counters, counters + count,
-                                              b->status_dev, batch_wait_cycles(), s);
+            le = sar::launch_batch_persistent(lists, s);
         b->launches = 1;
         e = cudaStreamEndCapture(s, &b->graph);
         if (e == cudaSuccess && le != cudaSuccess) e = le;
@@ -597,7 +663,7 @@ sar_status sar_batch_info(sar_batch b, sar_batch_info_t *info) {
     info->kernels_per_run = b->launches;
     info->range_classes = b->persistent ? b->n_range_classes : (int32_t)b->range.size();
     info->azimuth_classes = b->persistent ? b->n_az_classes : (int32_t)b->az.size();
-    info->work_bytes = b->persistent ? 0 : b->samples * 8;
+    info->work_bytes = b->persistent ? b->work_bytes : b->samples * 8;
     return SAR_OK;
 }
 

@@ -26,23 +26,39 @@ struct BItem {
     int32_t line0, nlines;
 };
 
-constexpr int kBatchThreads = 512;   // one block per SM
+constexpr int kBatchThreads = 512;       // one block per SM
+constexpr int kLongLines = 4;            // lines of a range item at least: a 32-byte sector of the image row
+constexpr int kBatchScratch = 3 * 16384; // samples of one block's scratch
+constexpr int kBatchNumLists = 5;        // range items of 512 and of 256 threads, all items of 128, azimuth items of 256, 512
 
-// Lines of length n that one item holds (the block's threads split into
-// groups of n / E threads, one line each), or 0 if n is not supported.
-int batch_lines_per_item(int n);
-// The name of the compiled schedule whose geometry the kernel uses for
-// length n (twiddle tables and filter order are built from it), or nullptr.
-const char *batch_schedule_name(int n);
-// Dynamic shared memory of one block.
-int batch_smem_bytes();
+// How the kernel runs lines of one length.
+struct BatchGeom {
+    const char *schedule;   // name of the compiled schedule of the same geometry; nullptr: length not supported
+    int threads;            // of a worker
+    int lines;              // that a worker holds at once
+    int set;                // lines of a range item that are stored together
+    bool parks;             // such a set needs the scratch
+};
+// whole_block: range items of 2048, 4096 and 8192 samples on all 512 threads.
+BatchGeom batch_geometry(int n, bool whole_block = false);
+
+// One launch: the items of list i are items[begin[i]] ... items[begin[i + 1]
+// - 1].  done[n_strips] and next[kBatchNumLists] must be zero (the caller
+// clears them before every launch); status is set to 5 when a bounded wait
+// runs out, and then nobody takes items any more.  scratch: batch_grid() *
+// kBatchScratch samples, or nullptr where no range item is longer than the
+// lines its worker holds.
+struct BatchLists {
+    const BItem *items;
+    int32_t begin[kBatchNumLists + 1];
+    const BStrip *strips;
+    int *done, *next, *status;
+    long long wait_cycles;
+    float2 *scratch;
+};
 // Blocks of the kernel resident on the whole current device (0 on error).
 int batch_grid();
-// One launch over the item list.  done[n_strips] and next[0] must be zero
-// (the caller clears them before every launch); status is set to 5 when a
-// bounded wait runs out, and then every block stops taking items.
-cudaError_t launch_batch_persistent(const BItem *items, int n_items, const BStrip *strips, int *done, int *next,
-                                    int *status, long long wait_cycles, cudaStream_t st);
+cudaError_t launch_batch_persistent(const BatchLists &lists, cudaStream_t st);
 cudaError_t prepare_batch_persistent();
 
 }  // namespace sar

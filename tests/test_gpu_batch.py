@@ -139,6 +139,43 @@ def test_one_launch_equals_multi_kernel_graph(sar):
     multi.destroy()
 
 
+@pytest.mark.parametrize("shapes", [
+    # azimuth lengths 512 ... 4096 side by side in the workers of a block, several lines per worker item,
+    # range items of 8192 and 16384 samples in two and four rounds with a remainder
+    [(4096, 2101), (4096, 1025), (8192, 613), (16384, 614), (2048, 1026), (4096, 2049)],
+    # azimuth lines of the whole block (8192, 16384) beside short ones, few items
+    [(256, 4097), (512, 9000), (8192, 3), (16384, 5), (16384, 1), (1024, 257)],
+    # several sets of short range lines per item, with a remainder
+    [(256, 16384), (512, 12001), (256, 3001)],
+], ids=["mixed_workers", "long_azimuth", "many_short"])
+def test_one_launch_mixed_lengths_equals_multi_kernel_graph(sar, shapes):
+    """Same engines, the corner turn a copy: bit-identical images, twice in a row."""
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    c64 = lambda *s: torch.randn(s, dtype=torch.complex64, device="cuda", generator=gen)
+    hr = {r: c64(r) for r, _ in shapes}
+    ha = {}
+    strips = []
+    for r, a in shapes:
+        L = max(256, 1 << (a - 1).bit_length())
+        ha.setdefault(L, c64(L))
+        strips.append(dict(n_range=r, n_az=a, raw=c64(a, r), range_spectrum=hr[r], az_spectrum=ha[L],
+                           image=torch.empty((r, a), dtype=torch.complex64, device="cuda")))
+    multi = sar.sar_batch_create(strips, flags=sar.SAR_BATCH_MULTI_KERNEL)
+    sar.sar_batch_run(multi)
+    sar.sar_sync()
+    want = [st["image"].clone() for st in strips]
+    multi.destroy()
+    one = sar.sar_batch_create(strips)
+    for _ in range(2):
+        for st in strips:
+            st["image"].fill_(float("nan"))
+        sar.sar_batch_run(one)
+        sar.sar_batch_status(one)
+        for st, w in zip(strips, want):
+            assert torch.equal(st["image"], w), (st["n_range"], st["n_az"])
+    one.destroy()
+
+
 def test_ragged_batch_wait_timeout_is_reported(sar):
     """A strip whose completion counter can never reach its target
     (host-side injection: one range line more expected than it has) makes the
