@@ -426,8 +426,9 @@ SAR_API sar_status sar_batch_destroy(sar_batch batch);
  * allocates its buffers from the server's stream-ordered memory pool, copies
  * its echo in from the device-resident pool scene of its class (the ingest,
  * part of its latency), runs sar_rda_process with its class's resident plan,
- * optionally copies the image out, frees its buffers and records a completion
- * event.  Requests on different slots overlap on the GPU.  When the oldest
+ * optionally delivers the image (the azimuth pass writes it into an output that
+ * is 16-byte aligned memory of the device, any other is copied to), frees its
+ * buffers and records a completion event.  Requests on different slots overlap on the GPU.  When the oldest
  * waiting request does not fit, later ones that do fit may pass it for at
  * most backfill_s seconds.  With size_priority set, each slot holds one
  * stream per distinct scene size, and a request runs on the one of its

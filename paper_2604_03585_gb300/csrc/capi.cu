@@ -631,14 +631,14 @@ sar_status sar_azimuth_compress(sar_plan p, void *data, sar_stream stream) {
     return run_fused(p, p->az, p->n_range, data, data, (cudaStream_t)stream, "azimuth compression launch");
 }
 
-// Range compression straight into the corner-turned image, then the
-// azimuth pass in place: two kernels.
-static sar_status run_folded(const sar_plan_s *p, const void *raw, void *image, cudaStream_t s) {
+// Range compression straight into the corner-turned image, then the azimuth
+// pass from image to out (in place where out is image): two kernels.
+static sar_status run_folded(const sar_plan_s *p, const void *raw, void *image, void *out, cudaStream_t s) {
     const SchedDesc &d = *p->range.sched;
     cudaError_t e = d.fused_ct((const float2 *)raw, (float2 *)image, p->n_az, p->n_range, p->n_az, p->range.filt,
                                p->range.tw, s);
     if (e != cudaSuccess) return cuda_fail(e, "range compression + corner turn launch");
-    return run_fused(p, p->az, p->n_range, image, image, s, "azimuth compression launch");
+    return run_fused(p, p->az, p->n_range, image, out, s, "azimuth compression launch");
 }
 
 static bool overlaps(const void *a, const void *b, size_t bytes) {
@@ -658,14 +658,15 @@ sar_status sar_corner_turn(sar_plan p, const void *in, void *out, sar_stream str
     return SAR_OK;
 }
 
-// The three passes into image [n_range][n_az] (raw clobbered when unfolded).
-static sar_status rda3(sar_plan p, void *raw, void *image, cudaStream_t s) {
+// The three passes into out [n_range][n_az], by way of image (out may be image;
+// raw clobbered when unfolded).
+static sar_status rda3(sar_plan p, void *raw, void *image, void *out, cudaStream_t s) {
     sar_status st;
-    if (p->fold) return run_folded(p, raw, image, s);
+    if (p->fold) return run_folded(p, raw, image, out, s);
     if ((st = run_fused(p, p->range, p->n_az, raw, raw, s, "range compression launch")) != SAR_OK) return st;
     cudaError_t e = sar::launch_transpose((const float2 *)raw, (float2 *)image, p->n_az, p->n_range, s);
     if (e != cudaSuccess) return cuda_fail(e, "corner turn launch");
-    return run_fused(p, p->az, p->n_range, image, image, s, "azimuth compression launch");
+    return run_fused(p, p->az, p->n_range, image, out, s, "azimuth compression launch");
 }
 
 sar_status sar_rda_process(sar_plan p, void *raw, void *image, sar_stream stream) {
@@ -677,12 +678,7 @@ sar_status sar_rda_process(sar_plan p, void *raw, void *image, sar_stream stream
         return fail(SAR_ERR_INVALID_ARG, "raw and image overlap");
     if (p->az_major)
         return fail(SAR_ERR_INVALID_ARG, "azimuth-major output needs a work buffer: use sar_rda_process_oop");
-    cudaStream_t s = (cudaStream_t)stream;
-    if (p->fold) return run_folded(p, raw, image, s);
-    if ((st = run_fused(p, p->range, p->n_az, raw, raw, s, "range compression launch")) != SAR_OK) return st;
-    cudaError_t e = sar::launch_transpose((const float2 *)raw, (float2 *)image, p->n_az, p->n_range, s);
-    if (e != cudaSuccess) return cuda_fail(e, "corner turn launch");
-    return run_fused(p, p->az, p->n_range, image, image, s, "azimuth compression launch");
+    return rda3(p, raw, image, image, (cudaStream_t)stream);
 }
 
 sar_status sar_range_compress_oop(sar_plan p, const void *in, void *out, sar_stream stream) {
@@ -741,7 +737,7 @@ sar_status sar_rda_process_oop(sar_plan p, const void *raw, void *work, void *im
         // the three passes leave the [n_range][n_az] image in work (image as
         // scratch when unfolded), then the fourth pass transposes it back
         if (p->fold) {
-            if ((st = run_folded(p, raw, work, s)) != SAR_OK) return st;
+            if ((st = run_folded(p, raw, work, work, s)) != SAR_OK) return st;
         } else {
             if ((st = run_fused(p, p->range, p->n_az, raw, image, s, "range compression launch")) != SAR_OK)
                 return st;
@@ -754,7 +750,7 @@ sar_status sar_rda_process_oop(sar_plan p, const void *raw, void *work, void *im
         if (e != cudaSuccess) return cuda_fail(e, "transpose back launch");
         return SAR_OK;
     }
-    if (p->fold) return run_folded(p, raw, image, s);
+    if (p->fold) return run_folded(p, raw, image, image, s);
     if ((st = run_fused(p, p->range, p->n_az, raw, work, s, "range compression launch")) != SAR_OK) return st;
     cudaError_t e = sar::launch_transpose((const float2 *)work, (float2 *)image, p->n_az, p->n_range, s);
     if (e != cudaSuccess) return cuda_fail(e, "corner turn launch");
@@ -995,7 +991,7 @@ static sar_status host_staging(sar_plan p, int sets) {
 static sar_status host_serial(sar_plan p, const void *raw, void *image, cudaStream_t s) {
     const size_t bytes = sizeof(float2) * (size_t)(p->n_az * p->n_range);
     SAR_CUDA(cudaMemcpyAsync(p->stage_raw[0], raw, bytes, cudaMemcpyHostToDevice, s), "host-to-device copy");
-    sar_status st = rda3(p, p->stage_raw[0], p->stage_img[0], s);
+    sar_status st = rda3(p, p->stage_raw[0], p->stage_img[0], p->stage_img[0], s);
     if (st != SAR_OK) return st;
     const void *result = p->stage_img[0];
     if (p->az_major) {   // the fourth pass, into the staged raw echo (no longer needed)
@@ -1152,3 +1148,12 @@ sar_status sar_sync(sar_stream stream) {
 }
 
 }  // extern "C"
+
+namespace sar {
+// sar_rda_process with the azimuth pass writing its result to out instead of
+// image (internal: valid, 16-byte aligned device buffers that do not overlap,
+// a plan without azimuth-major output).
+sar_status rda_process_into(sar_plan p, void *raw, void *image, void *out, cudaStream_t s) {
+    return rda3(p, raw, image, out, s);
+}
+}  // namespace sar

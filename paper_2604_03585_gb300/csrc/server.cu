@@ -30,6 +30,7 @@
 namespace sar {
 sar_status report_error(sar_status st, const char *msg);
 sar_status validate_device_ptr(const void *p, const char *what);
+sar_status rda_process_into(sar_plan p, void *raw, void *image, void *out, cudaStream_t s);
 }  // namespace sar
 
 namespace {
@@ -50,6 +51,18 @@ struct Class {
     int level = 0;   // index of the slot stream its requests run on
     size_t bytes() const { return (size_t)n_range * (size_t)n_az * 8; }
 };
+
+// Whether a kernel's 16-byte aligned accesses can go to p: memory of this
+// device (any other output is copied to).
+bool kernel_can_write(const void *p, int device) {
+    cudaPointerAttributes a;
+    if ((uintptr_t)p & 15u) return false;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == device;
+}
 
 }  // namespace
 
@@ -176,6 +189,8 @@ sar_status sar_server_run(sar_server s, const sar_request *reqs, int32_t n, int3
         res[i] = sar_request_result{mode == SAR_SERVE_CLOSED_LOOP ? 0.0 : reqs[i].arrival_s, -1.0, -1.0, -1};
     }
     using clock = std::chrono::steady_clock;
+    int device = 0;
+    cudaGetDevice(&device);
     if (cudaDeviceSynchronize() != cudaSuccess) return sar::report_error(SAR_ERR_CUDA, "device not idle");
     cudaEventRecord(s->base, s->slots[0].streams[0]);
     cudaEventSynchronize(s->base);
@@ -200,9 +215,13 @@ sar_status sar_server_run(sar_server s, const sar_request *reqs, int32_t n, int3
         }
         res[i].admit_s = now_s();
         bool ok = cudaMemcpyAsync(raw, c.pool, bytes, cudaMemcpyDeviceToDevice, st) == cudaSuccess;
-        ok = ok && sar_rda_process(c.plan, raw, img, st) == SAR_OK;
-        if (ok && reqs[i].output)
-            ok = cudaMemcpyAsync(reqs[i].output, img, bytes, cudaMemcpyDeviceToDevice, st) == cudaSuccess;
+        // the azimuth pass writes the image where it is wanted, which saves the
+        // copy out and its 16 bytes of traffic per sample; out of place, so
+        // that requests of one class may share an output as with the copy
+        void *out = reqs[i].output;
+        const bool direct = out && kernel_can_write(out, device);
+        ok = ok && sar::rda_process_into(c.plan, raw, img, direct ? out : img, st) == SAR_OK;
+        if (ok && out && !direct) ok = cudaMemcpyAsync(out, img, bytes, cudaMemcpyDeviceToDevice, st) == cudaSuccess;
         cudaFreeAsync(raw, st);
         cudaFreeAsync(img, st);
         ok = ok && cudaEventRecord(sl.done, st) == cudaSuccess;

@@ -61,6 +61,26 @@ def test_results_are_the_same_alone_and_in_the_mix(sar, classes, size_priority, 
     srv.destroy()
 
 
+@pytest.mark.parametrize("offset", [0, 1], ids=["aligned", "copied"])
+def test_outputs_written_directly_copied_or_shared(sar, classes, offset):
+    """The azimuth pass writes an aligned output itself and one that is only 8-byte aligned is copied to;
+    requests of one class may share an output."""
+    srv = sar.sar_server_create(classes, hbm_budget_bytes=1 << 30, max_inflight=8)
+    c = classes[1]
+    want = _outputs(classes, [1])[0]
+    sar.sar_server_run(srv, [(0.0, 1, want)], mode=sar.SAR_SERVE_CLOSED_LOOP)
+    n = c["n_range"] * c["n_az"]
+    flat = [torch.full((n + 2,), float("nan"), dtype=torch.complex64, device="cuda") for _ in range(3)]
+    outs = [flat[i % 3][offset:offset + n] for i in range(12)]        # three buffers, four requests each
+    res = sar.sar_server_run(srv, [(0.0, 1, o) for o in outs], mode=sar.SAR_SERVE_CLOSED_LOOP)
+    assert all(r["status"] == 0 for r in res)
+    for f in flat:
+        assert torch.equal(f[offset:offset + n].view(c["n_range"], c["n_az"]), want)
+        rest = torch.cat([f[:offset], f[offset + n:]])
+        assert torch.isnan(rest.real).all()                            # nothing beside the image
+    srv.destroy()
+
+
 def test_server_images_match_oracle(sar, classes):
     orc = oracle.default()
     srv = sar.sar_server_create(classes, hbm_budget_bytes=1 << 30, max_inflight=4)
