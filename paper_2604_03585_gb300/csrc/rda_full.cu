@@ -30,19 +30,71 @@ struct RdColumn {
     float mig_hi, mig_lo;   // 1 / D(f_j) - 1 = mig_hi + mig_lo
 };
 
-// cos and sin of 2 pi t / 16 for the taps t = -7 ... 8 (index t + 7),
-// evaluated at compile time
-#define SAR_RC(t) float2{(float)ct::cos2pi(t, 16), (float)ct::sin2pi(t, 16)}
-__constant__ float2 kHann16[16] = {SAR_RC(-7), SAR_RC(-6), SAR_RC(-5), SAR_RC(-4), SAR_RC(-3), SAR_RC(-2),
-                                   SAR_RC(-1), SAR_RC(0),  SAR_RC(1),  SAR_RC(2),  SAR_RC(3),  SAR_RC(4),
-                                   SAR_RC(5),  SAR_RC(6),  SAR_RC(7),  SAR_RC(8)};
-#undef SAR_RC
+// The interpolation weights h(x) = sinc(x) (1 + cos(2 pi x / 16)) / 2 at the 16
+// taps t = -7 ... 8 of a source position k0 + frac, as polynomials in u = frac -
+// 1/2.  h is even, so taps t and 1 - t are h(u + 1/2 - t) = E_t(u^2) + u
+// O_t(u^2) and E_t(u^2) - u O_t(u^2): ten fused multiply-adds give both.  E_t
+// and O_t are interpolated in v = u^2 at five Chebyshev points of [0, 1/4]
+// (Newton's divided differences, expanded), at compile time in FP64: the
+// largest error of a weight is 1.2e-9, and 9e-8 in FP32 arithmetic, all of it
+// rounding, with an RMS of 2.5e-8 at the central taps and below 1e-8 beyond.
+namespace rcw {
+// a * b + c, two-wide: one packed instruction, each half rounded as fmaf
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_pack(a)), "l"(f2_pack(b)), "l"(f2_pack(c)));
+    return f2_unpack(r);
+}
+constexpr int K = 5;
+__host__ __device__ constexpr double weight(double x) {
+    const double ax = x < 0 ? -x : x;
+    const double turns = ax * 0.5 - (double)(long long)(ax * 0.5);   // of pi x
+    const double sinc = ax == 0 ? 1.0 : ct::sin2pi_f(turns) / (ct::kPi * ax);
+    return sinc * 0.5 * (1.0 + ct::cos2pi_f(ax / 16.0));
+}
+struct Poly {
+    double c[K];   // of v^0 ... v^4
+};
+// ODD: O_t, else E_t
+__host__ __device__ constexpr Poly fit(int t, bool odd) {
+    double v[K] = {}, d[K] = {};
+    for (int i = 0; i < K; ++i) {
+        const double u = 0.5 * ct::cos2pi_f((2 * i + 1) / (8.0 * K));
+        const double p = weight(u + 0.5 - t), m = weight(-u + 0.5 - t);
+        v[i] = u * u;
+        d[i] = odd ? (p - m) / (2.0 * u) : (p + m) * 0.5;
+    }
+    for (int k = 1; k < K; ++k)
+        for (int i = K - 1; i >= k; --i) d[i] = (d[i] - d[i - 1]) / (v[i] - v[i - k]);
+    Poly r = {};
+    for (int k = K - 1; k >= 0; --k) {   // r <- r (x - v[k]) + d[k]
+        for (int i = K - 1; i > 0; --i) r.c[i] = r.c[i - 1] - v[k] * r.c[i];
+        r.c[0] = d[k] - v[k] * r.c[0];
+    }
+    return r;
+}
+// the polynomial at two v by Horner's rule
+template <int T, bool ODD>
+__device__ __forceinline__ float2 at(float2 v) {
+    constexpr Poly p = fit(T, ODD);
+    float2 r = make_float2((float)p.c[K - 1], (float)p.c[K - 1]);
+#pragma unroll
+    for (int i = K - 2; i >= 0; --i) r = fma2(r, v, make_float2((float)p.c[i], (float)p.c[i]));
+    return r;
+}
+}  // namespace rcw
 
 // RCMC tiles: 32 frequency columns (one per lane) x 128 range bins per block of
 // 8 warps.  A block stages the input rows its outputs touch in shared memory
 // (rows n0 + min shift - 7 ... n0 + 127 + max shift + 8, zero outside the
 // scene); the host sizes that span from the geometry, and a block whose span
 // does not fit reads global memory directly.
+// Bound by ALU issue: 178 thread instructions per output (223 with the weights
+// from reciprocals and sines; the floor of the 4096 x 4096 scene's 268 MB is 40
+// us, of its instructions 74).  102.8 us at 4096 x 4096, from 122.5: polynomial
+// weights for two outputs at once 105.0 (one at a time 123.5, four 108.8, with
+// the coefficients in constant memory 144), rows staged by asynchronous copies
+// 102.8.  Tiles of 64 and 256 bins: 107.9 and 106.6.
 constexpr int kRcCols = 32;
 constexpr int kRcRows = 128;
 constexpr int kRcWarps = 8;
@@ -65,67 +117,46 @@ __device__ __forceinline__ void rc_locate(int n, const RdColumn& c, float rn_hi,
     if (frac >= 1.f) { frac -= 1.f; k0 += 1; }
 }
 
-__device__ __forceinline__ float rc_rcp(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-// (cw, sw) = (cos, sin)(pi frac / 8) and s = sin(pi frac) for frac in (0, 1),
-// each to a few FP32 ulps, s relative to its own size near frac = 0 and 1.
-// With g = min(frac, 1 - frac) <= 1/2 and theta = pi g / 8 <= pi / 16, sin and
-// cos of theta come from their Taylor series (the first omitted terms are below
-// 2e-12), s = sin(pi g) = sin(8 theta) from three angle doublings in which
-// every cosine stays >= cos(pi / 4) (no cancellation), and for frac > 1/2 the
-// window angle is pi / 8 - theta.
-__device__ __forceinline__ void rc_trig(float frac, float& cw, float& sw, float& s) {
-    const bool flip = frac > 0.5f;
-    const float g = flip ? 1.f - frac : frac;   // exact
-    const float th = g * 0.392699081698724155f;  // pi / 8
-    const float t2 = th * th;
-    const float s8 = th * fmaf(t2, fmaf(t2, fmaf(t2, -1.f / 5040.f, 1.f / 120.f), -1.f / 6.f), 1.f);
-    const float c8 = fmaf(t2, fmaf(t2, fmaf(t2, fmaf(t2, 1.f / 40320.f, -1.f / 720.f), 1.f / 24.f), -0.5f), 1.f);
-    float a = 2.f * s8;
-    const float s4 = a * c8, c4 = fmaf(-a, s8, 1.f);   // pi g / 4
-    a = 2.f * s4;
-    const float s2 = a * c4, c2 = fmaf(-a, s4, 1.f);   // pi g / 2
-    s = 2.f * s2 * c2;                                   // pi g
-    constexpr float C = 0.923879532511286756f, S = 0.382683432365089772f;   // cos, sin of pi / 8
-    cw = flip ? fmaf(C, c8, S * s8) : c8;
-    sw = flip ? fmaf(S, c8, -C * s8) : s8;
-}
-
-// The 16 taps at source position k0 + frac, rows read through row(t) for
-// t = -7 ... 8.  Weight h_t = sinc(x) w(x), x = frac - t,
-// w(x) = 0.5 (1 + cos(2 pi x / 16)).  With sin(pi x) = (-1)^t sin(pi frac) and
-// cos(2 pi x / 16) = cw cos_t + sw sin_t = u_t, cos_t, sin_t the cos and sin of
-// 2 pi t / 16:
-//   h_t = (sin(pi frac) / (2 pi)) (-1)^t (1 + u_t) / x.
-// Taps t and t + 8 share (-1)^t and have u_{t+8} = -u_t.
-template <class Row>
-__device__ __forceinline__ float2 rc_interp(float frac, Row row) {
-    if (frac == 0.f) return row(0);   // h_0 = 1, every other tap sits on a zero of the sinc
-    float cw, sw, s;
-    rc_trig(frac, cw, sw, s);
-    float2 acc = make_float2(0.f, 0.f);
+// The 16 taps at kRcWide source positions k0 + frac[j], rows of position j read
+// through row(j, t) for t = -7 ... 8, outer pairs first.  Positions go through
+// the polynomials together, two to a packed instruction, because every
+// coefficient costs a move into a register pair whatever uses it.
+constexpr int kRcWide = 2;
+template <int T, class Row>
+__device__ __forceinline__ void rc_pairs(const float2 (&u)[kRcWide / 2], const float2 (&v)[kRcWide / 2],
+                                         float2 (&acc)[kRcWide], Row& row) {
+    float2 h[kRcWide / 2][2];
 #pragma unroll
-    for (int t = -7; t <= 0; ++t) {
-        const float2 cs = kHann16[t + 7];
-        const float u = fmaf(cw, cs.x, sw * cs.y);
-        const float r1 = rc_rcp(frac - (float)t), r2 = rc_rcp(frac - (float)(t + 8));
-        float h1 = fmaf(u, r1, r1), h2 = fmaf(-u, r2, r2);
-        if (t & 1) {
-            h1 = -h1;
-            h2 = -h2;
-        }
-        const float2 v1 = row(t), v2 = row(t + 8);
-        acc.x = fmaf(h1, v1.x, acc.x);
-        acc.y = fmaf(h1, v1.y, acc.y);
-        acc.x = fmaf(h2, v2.x, acc.x);
-        acc.y = fmaf(h2, v2.y, acc.y);
+    for (int i = 0; i < kRcWide / 2; ++i) {
+        const float2 e = rcw::at<T, false>(v[i]), o = rcw::at<T, true>(v[i]);
+        h[i][0] = rcw::fma2(u[i], o, e);
+        h[i][1] = rcw::fma2(make_float2(-u[i].x, -u[i].y), o, e);
     }
-    const float a = s * 0.159154943091895336f;   // sin(pi frac) / (2 pi)
-    return make_float2(acc.x * a, acc.y * a);
+#pragma unroll
+    for (int j = 0; j < kRcWide; ++j) {
+        const float h1 = j & 1 ? h[j / 2][0].y : h[j / 2][0].x, h2 = j & 1 ? h[j / 2][1].y : h[j / 2][1].x;
+        const float2 v1 = row(j, T), v2 = row(j, 1 - T);
+        acc[j].x = fmaf(h1, v1.x, acc[j].x);
+        acc[j].y = fmaf(h1, v1.y, acc[j].y);
+        acc[j].x = fmaf(h2, v2.x, acc[j].x);
+        acc[j].y = fmaf(h2, v2.y, acc[j].y);
+    }
+    if constexpr (T < 0) rc_pairs<T + 1>(u, v, acc, row);
+}
+template <class Row>
+__device__ __forceinline__ void rc_interp(const float (&frac)[kRcWide], float2 (&acc)[kRcWide], Row row) {
+    float2 u[kRcWide / 2], v[kRcWide / 2];
+#pragma unroll
+    for (int i = 0; i < kRcWide / 2; ++i) {
+        u[i] = make_float2(frac[2 * i] - 0.5f, frac[2 * i + 1] - 0.5f);
+        v[i] = make_float2(u[i].x * u[i].x, u[i].y * u[i].y);
+    }
+#pragma unroll
+    for (int j = 0; j < kRcWide; ++j) acc[j] = make_float2(0.f, 0.f);
+    rc_pairs<-7>(u, v, acc, row);
+#pragma unroll
+    for (int j = 0; j < kRcWide; ++j)
+        if (frac[j] == 0.f) acc[j] = row(j, 0);   // h_0 = 1, every other tap sits on a zero of the sinc
 }
 
 __global__ void __launch_bounds__(kRcCols * kRcWarps)
@@ -153,31 +184,42 @@ rcmc_tile_kernel(const float2* __restrict__ in, float2* __restrict__ out, int n_
     const int span = hi - lo + 1;
     const bool staged = span <= staged_rows;
     if (staged) {
+        // copied without a stop in registers, all of a thread's rows in flight
+        // (src size 0: zeros outside the scene)
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(tile) + lane * 8;
 #pragma unroll 4
         for (int rr = warp; rr < span; rr += kRcWarps) {
             const int k = lo + rr;
-            tile[rr * kRcCols + lane] =
-                (jok && k >= 0 && k < n_range) ? in[(int64_t)k * n_f + j] : make_float2(0.f, 0.f);
+            const bool inside = jok && k >= 0 && k < n_range;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst + rr * (kRcCols * 8)),
+                         "l"(in + (inside ? (int64_t)k * n_f + j : 0)), "r"(inside ? 8 : 0)
+                         : "memory");
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
     }
     if (!jok) return;
-    for (int n = n0 + warp; n <= n1; n += kRcWarps) {
-        int k0;
-        float frac;
-        rc_locate(n, c, rn_hi, rn_lo, k0, frac);
-        float2 y;
+    for (int n = n0 + warp; n <= n1; n += kRcWide * kRcWarps) {
+        int k0[kRcWide];
+        float frac[kRcWide];
+        float2 y[kRcWide];
+#pragma unroll
+        for (int i = 0; i < kRcWide; ++i) rc_locate(min(n + i * kRcWarps, n1), c, rn_hi, rn_lo, k0[i], frac[i]);
         if (staged) {
-            k0 = min(max(k0, lo + 7), hi - 8);   // already within; keeps every read inside the tile
-            const float2* b = tile + (k0 - lo) * kRcCols + lane;
-            y = rc_interp(frac, [&](int t) { return b[t * kRcCols]; });
+            const float2* b[kRcWide];
+#pragma unroll
+            for (int i = 0; i < kRcWide; ++i)   // already within; keeps every read inside the tile
+                b[i] = tile + (min(max(k0[i], lo + 7), hi - 8) - lo) * kRcCols + lane;
+            rc_interp(frac, y, [&](int i, int t) { return b[i][t * kRcCols]; });
         } else {
-            y = rc_interp(frac, [&](int t) {
-                const int k = k0 + t;
+            rc_interp(frac, y, [&](int i, int t) {
+                const int k = k0[i] + t;
                 return (k >= 0 && k < n_range) ? in[(int64_t)k * n_f + j] : make_float2(0.f, 0.f);
             });
         }
-        __stcs(out + (int64_t)n * n_f + j, y);
+#pragma unroll
+        for (int i = 0; i < kRcWide; ++i)
+            if (n + i * kRcWarps <= n1) __stcs(out + (int64_t)(n + i * kRcWarps) * n_f + j, y[i]);
     }
 }
 
@@ -194,7 +236,7 @@ rcmc_tile_kernel(const float2* __restrict__ in, float2* __restrict__ out, int n_
 // conj(FFT(conj .)) (Sec. II-C).  Otherwise the forward FFT of the line (the
 // Range-Doppler domain, Sec. IV-A step 2).
 template <class SC, bool COMPRESS>
-__global__ void __launch_bounds__(SC::T, min_blocks_128<SC, 1>())
+__global__ void __launch_bounds__(SC::T, SC::T >= 256 ? min_blocks_128<SC, 1>() : 0)
 az_streamed_kernel(const float2* in, float2* out, int64_t n_lines, const float2* tw, const RdColumn* cols,
                    double r_near) {
     extern __shared__ float2 smem_dyn[];
