@@ -536,6 +536,8 @@ sar_status sar_autotune(int64_t n, int64_t n_lines, int32_t reps, int32_t kind, 
         if ((e = d.prepare()) != cudaSuccess) break;
         float2 *tw = tab + n, *filt = tab;
         if ((e = sar::build_twiddles(d, tw, s)) != cudaSuccess) break;
+        // a kernel may read its tables before its predecessor on the stream is done
+        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
         auto run = [&]() {
             return ct ? d.fused_ct(in, outb, n_lines, n, n_lines, filt, tw, s)
                       : d.fused(in, outb, n_lines, n, (int)n, filt, tw, ctl, s);

@@ -39,10 +39,41 @@ cudaError_t prepare_sched() {
     return cudaFuncSetAttribute(dft_lines_kernel<SC, LPB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
+// Few short lines (up to four warps per SM of 152) take the kernels made for
+// latency, launched programmatically behind the stream's last kernel.
+template <class SC>
+constexpr bool has_small_kernel() {
+    return SC::P == 2 && SC::MINB == 0 && SC::E <= 32 && SC::T <= 32;
+}
+template <class SC>
+bool small_launch(int64_t n_lines) {
+    return n_lines * SC::T <= 608 * 32;
+}
+template <class K, class... Args>
+cudaError_t launch_behind(K kernel, unsigned blocks, unsigned threads, int smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 template <class SC, int LPB>
 cudaError_t launch_fused(const float2 *in, float2 *out, int64_t n_lines, int64_t ld, int valid,
                          const float2 *filt, const float2 *tw, const FusedCtl &, cudaStream_t st) {
     if (n_lines <= 0) return cudaSuccess;
+    if constexpr (has_small_kernel<SC>()) {
+        constexpr int L = small_lines_per_block<SC>();
+        if (valid == SC::N && small_launch<SC>(n_lines))
+            return launch_behind(fused_small_kernel<SC>, (unsigned)((n_lines + L - 1) / L), SC::T * L,
+                                 smem_bytes_of<SC, L>(), st, in, out, n_lines, ld, filt, tw);
+    }
     const int64_t blocks = (n_lines + LPB - 1) / LPB;
     constexpr int smem = smem_bytes_of<SC, LPB>();
     const unsigned grid = (unsigned)blocks, threads = SC::T * LPB;
@@ -213,6 +244,11 @@ cudaError_t launch_range_ct(const float2 *in, float2 *img, int64_t n_lines, int6
                             const float2 *filt, const float2 *tw, cudaStream_t st) {
     if (n_lines <= 0) return cudaSuccess;
     if (n_lines % QL) return cudaErrorInvalidValue;
+    if constexpr (has_small_kernel<SC>()) {
+        if (small_launch<SC>(n_lines))
+            return launch_behind(fused_range_ct_small_kernel<SC, QL>, (unsigned)(n_lines / QL), SC::T * QL,
+                                 ct_smem_bytes<SC, QL>(), st, in, img, ld_in, ld_img, filt, tw);
+    }
     fused_range_ct_kernel<SC, QL, ROLL><<<(unsigned)(n_lines / QL), SC::T * QL, ct_smem_bytes<SC, QL>(), st>>>(
         in, img, n_lines, ld_in, ld_img, filt, tw);
     return cudaGetLastError();

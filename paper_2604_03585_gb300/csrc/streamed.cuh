@@ -229,6 +229,34 @@ fused_seg_kernel(const Seg* segs, const int64_t* line_begin, int n_seg, int64_t 
     }
 }
 
+// The lines of a block, in pass-1 geometry, stored transposed: natural order
+// into shared memory, then one QL*8-byte chunk per range bin.
+template <class SC, int QL>
+__device__ __forceinline__ void store_corner_turned(const float2 (&v)[SC::E], float2* smem_dyn, int t, int lib,
+                                                    float2* img, int64_t ld_img, int64_t a0) {
+    constexpr int R1 = SC::R1, S1 = SC::S1, G1 = SC::E / R1;
+    float2* sm = smem_dyn + lib * SC::SMEM_ELEMS;
+    line_sync<SC, QL>(lib);
+#pragma unroll
+    for (int s = 0; s < G1; ++s) {
+        const int lo = t + SC::T * s;
+#pragma unroll
+        for (int r = 0; r < R1; ++r) sm[lo + r * S1] = v[s * R1 + r];
+    }
+    __syncthreads();
+    // ---- transposed store: one QL*8-byte chunk per range bin
+    static_assert(QL == 2 || QL == 4, "chunks of two or four complex64");
+    for (int n = threadIdx.x; n < SC::N; n += SC::T * QL) {
+        float4* dst = reinterpret_cast<float4*>(img + (int64_t)n * ld_img + a0);
+        const float2 c0 = smem_dyn[n], c1 = smem_dyn[SC::SMEM_ELEMS + n];
+        dst[0] = make_float4(c0.x, c0.y, c1.x, c1.y);
+        if constexpr (QL == 4) {
+            const float2 c2 = smem_dyn[2 * SC::SMEM_ELEMS + n], c3 = smem_dyn[3 * SC::SMEM_ELEMS + n];
+            dst[1] = make_float4(c2.x, c2.y, c3.x, c3.y);
+        }
+    }
+}
+
 // Range compression with the corner turn folded into its store (the
 // paper's Sec. IV-A steps 1 and 2 in one kernel).  A block compresses QL
 // consecutive range lines a0 .. a0+QL-1 (QL = 4); after the inverse pass the
@@ -257,25 +285,25 @@ __device__ __forceinline__ void fused_range_ct_body(const float2* in, float2* im
 #pragma unroll
         for (int r = 0; r < R1; ++r) v[s * R1 + r] = x[r];
     }
-    line_sync<SC, QL>(lib);
-#pragma unroll
-    for (int s = 0; s < G1; ++s) {
-        const int lo = t + SC::T * s;
-#pragma unroll
-        for (int r = 0; r < R1; ++r) sm[lo + r * S1] = v[s * R1 + r];
-    }
-    __syncthreads();
-    // ---- transposed store: one QL*8-byte chunk per range bin
-    static_assert(QL == 2 || QL == 4, "chunks of two or four complex64");
-    for (int n = threadIdx.x; n < SC::N; n += SC::T * QL) {
-        float4* dst = reinterpret_cast<float4*>(img + (int64_t)n * ld_img + a0);
-        const float2 c0 = smem_dyn[n], c1 = smem_dyn[SC::SMEM_ELEMS + n];
-        dst[0] = make_float4(c0.x, c0.y, c1.x, c1.y);
-        if constexpr (QL == 4) {
-            const float2 c2 = smem_dyn[2 * SC::SMEM_ELEMS + n], c3 = smem_dyn[3 * SC::SMEM_ELEMS + n];
-            dst[1] = make_float4(c2.x, c2.y, c3.x, c3.y);
-        }
-    }
+    store_corner_turned<SC, QL>(v, smem_dyn, t, lib, img, ld_img, a0);
+}
+
+// The same for a few short lines (fused_small_kernel).
+template <class SC, int QL>
+__global__ void __launch_bounds__(SC::T* QL)
+fused_range_ct_small_kernel(const float2* in, float2* img, int64_t ld_in, int64_t ld_img, const float2* filt,
+                            const float2* tw) {
+    extern __shared__ float2 smem_dyn[];
+    grid_release_dependents();
+    const int lib = threadIdx.x / SC::T, t = threadIdx.x % SC::T;
+    const int64_t a0 = (int64_t)blockIdx.x * QL;
+    SmallTables<SC> tab;
+    tab.load(filt, tw, t);
+    grid_wait_predecessor();
+    float2 v[SC::E];
+    global_load<SC, false>(in + (a0 + lib) * ld_in, SC::N, t, v);
+    small_compress<SC, QL>(v, tab, smem_dyn + lib * SC::SMEM_ELEMS, t, lib);
+    store_corner_turned<SC, QL>(v, smem_dyn, t, lib, img, ld_img, a0);
 }
 
 // The fold whose image tiles leave through the tensor memory accelerator:

@@ -258,6 +258,44 @@ def test_folded_corner_turn_matches_unfolded(sar, orc, name):
     plain.destroy()
 
 
+@pytest.mark.parametrize("n_range,n_az", [(256, 256), (256, 1216), (256, 1220), (512, 4), (512, 608), (1024, 37),
+                                          (1024, 608), (1024, 612)])
+def test_small_scenes_match_large_ones(sar, n_range, n_az):
+    """Few short lines take the kernels made for latency (here on both sides of their limit, and with a
+    remainder in the last block): bit-identical to the same lines at the head of a larger array.  Launched
+    back to back and from a captured graph, each behind its predecessor on the stream."""
+    gen = torch.Generator(device="cuda").manual_seed(n_range + n_az)
+    c64 = lambda *s: torch.randn(s, dtype=torch.complex64, device="cuda", generator=gen)
+    hr, ha, raw = c64(n_range), c64(512), c64(4096, n_range)
+    small = sar.sar_plan_create(n_range, n_az, hr, c64(n_az))
+    large = sar.sar_plan_create(n_range, 4096, hr, c64(4096))
+    want, out = empty_c64(4096, n_range), empty_c64(n_az, n_range)
+    sar.sar_range_compress_oop(large, raw, want)
+    sar.sar_range_compress_oop(small, raw, out)
+    assert torch.equal(out, want[:n_az])
+    data = raw[:n_az].clone()                                    # in place, twice in a row
+    sar.sar_range_compress(small, data)
+    assert torch.equal(data, out)
+    if n_az % 4 == 0:                                            # folded: the same, corner-turned
+        assert sar.sar_plan_folds_corner_turn(small)
+        image = empty_c64(n_range, n_az)
+        sar.sar_range_compress_ct(small, raw, image)
+        assert torch.equal(image, out.t())
+    if n_az in (256, 608):
+        image, work, again = empty_c64(n_range, n_az), empty_c64(n_range, n_az), empty_c64(n_range, n_az)
+        sar.sar_rda_process_oop(small, raw, work, image)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            for _ in range(3):
+                sar.sar_rda_process_oop(small, raw, work, again)
+        for _ in range(2):
+            again.fill_(float("nan"))
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(again, image)
+
+
 @pytest.mark.parametrize("n_range,n_az", [(4096, 36), (2048, 100), (8192, 12), (4096, 300), (2048, 260)])
 def test_folded_corner_turn_at_narrow_images(sar, n_range, n_az):
     """The default folded range pass writes its image tiles as tensor-store
