@@ -9,6 +9,8 @@
 // Pure data movement: bit-exact.
 #include <atomic>
 
+#include "launch_behind.h"
+#include "sar_common.cuh"
 #include "tables.h"
 
 namespace sar {
@@ -17,9 +19,10 @@ constexpr int kTile = 32;
 constexpr int kRowsPerPass = 8;   // block = 32 x 8 threads, 4 elements each way
 
 __global__ void __launch_bounds__(kTile * kRowsPerPass)
-corner_turn_kernel(const float2 *__restrict__ in, float2 *__restrict__ out, int64_t rows, int64_t cols,
+corner_turn_kernel(const float2 *in, float2 *__restrict__ out, int64_t rows, int64_t cols,
                    int64_t tiles_c) {
     __shared__ float2 tile[kTile][kTile + 1];
+    grid_enter();
     const int64_t tr = blockIdx.x / tiles_c;           // tile row (over `rows`)
     const int64_t tc = blockIdx.x % tiles_c;           // tile column (over `cols`)
     const int tx = threadIdx.x % kTile, ty = threadIdx.x / kTile;
@@ -50,9 +53,10 @@ constexpr int kBig = 64;
 __device__ __forceinline__ int ct_chunk(int r, int j) { return r * 32 + (j ^ ((r >> 1) & 7)); }
 
 __global__ void __launch_bounds__(256)
-corner_turn64_kernel(const float4 *__restrict__ in, float4 *__restrict__ out, int64_t rows, int64_t cols,
+corner_turn64_kernel(const float4 *in, float4 *__restrict__ out, int64_t rows, int64_t cols,
                      int64_t tiles_c) {
     __shared__ float4 tile[kBig * 32];                 // 64 rows x 32 chunks of 16 B
+    grid_enter();
     const int64_t tr = blockIdx.x / tiles_c, tc = blockIdx.x % tiles_c;
     const int64_t r0 = tr * kBig, c0 = tc * kBig;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -90,14 +94,12 @@ cudaError_t launch_transpose(const float2 *in, float2 *out, int64_t rows, int64_
     if (variant != 1 && rows % kBig == 0 && cols % kBig == 0 && ((uintptr_t)in & 15) == 0 &&
         ((uintptr_t)out & 15) == 0 && variant == 2) {
         const int64_t tiles_c = cols / kBig, blocks = (rows / kBig) * tiles_c;
-        corner_turn64_kernel<<<(unsigned)blocks, 256, 0, st>>>((const float4 *)in, (float4 *)out, rows, cols,
-                                                                tiles_c);
-        return cudaGetLastError();
+        return launch_behind(corner_turn64_kernel, blocks, 256, 0, 1, st, (const float4 *)in, (float4 *)out, rows, cols,
+                             tiles_c);
     }
     const int64_t tiles_r = (rows + kTile - 1) / kTile, tiles_c = (cols + kTile - 1) / kTile;
     const int64_t blocks = tiles_r * tiles_c;
-    corner_turn_kernel<<<(unsigned)blocks, kTile * kRowsPerPass, 0, st>>>(in, out, rows, cols, tiles_c);
-    return cudaGetLastError();
+    return launch_behind(corner_turn_kernel, blocks, kTile * kRowsPerPass, 0, 1, st, in, out, rows, cols, tiles_c);
 }
 
 }  // namespace sar

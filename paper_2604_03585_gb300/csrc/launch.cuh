@@ -2,6 +2,7 @@
 // instantiation units).
 #pragma once
 
+#include "launch_behind.h"
 #include "persistent.cuh"
 #include "streamed.cuh"
 #include "registry.h"
@@ -49,21 +50,6 @@ template <class SC>
 bool small_launch(int64_t n_lines) {
     return n_lines * SC::T <= 608 * 32;
 }
-template <class K, class... Args>
-cudaError_t launch_behind(K kernel, unsigned blocks, unsigned threads, int smem, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks, 1, 1);
-    cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 template <class SC, int LPB>
 cudaError_t launch_fused(const float2 *in, float2 *out, int64_t n_lines, int64_t ld, int valid,
                          const float2 *filt, const float2 *tw, const FusedCtl &, cudaStream_t st) {
@@ -71,24 +57,20 @@ cudaError_t launch_fused(const float2 *in, float2 *out, int64_t n_lines, int64_t
     if constexpr (has_small_kernel<SC>()) {
         constexpr int L = small_lines_per_block<SC>();
         if (valid == SC::N && small_launch<SC>(n_lines))
-            return launch_behind(fused_small_kernel<SC>, (unsigned)((n_lines + L - 1) / L), SC::T * L,
-                                 smem_bytes_of<SC, L>(), st, in, out, n_lines, ld, filt, tw);
+            return launch_behind(fused_small_kernel<SC>, (n_lines + L - 1) / L, SC::T * L, smem_bytes_of<SC, L>(), 1,
+                                 st, in, out, n_lines, ld, filt, tw);
     }
     const int64_t blocks = (n_lines + LPB - 1) / LPB;
     constexpr int smem = smem_bytes_of<SC, LPB>();
-    const unsigned grid = (unsigned)blocks, threads = SC::T * LPB;
-    if constexpr (SC::MINB > 0) {
-        if (valid < SC::N)
-            fused_compress_kernel_capped<SC, LPB, true><<<grid, threads, smem, st>>>(in, out, n_lines, ld, valid, filt, tw);
-        else
-            fused_compress_kernel_capped<SC, LPB, false><<<grid, threads, smem, st>>>(in, out, n_lines, ld, valid, filt, tw);
-    } else {
-        if (valid < SC::N)
-            fused_compress_kernel<SC, LPB, true><<<grid, threads, smem, st>>>(in, out, n_lines, ld, valid, filt, tw);
-        else
-            fused_compress_kernel<SC, LPB, false><<<grid, threads, smem, st>>>(in, out, n_lines, ld, valid, filt, tw);
-    }
-    return cudaGetLastError();
+    constexpr int threads = SC::T * LPB;
+    if constexpr (SC::MINB > 0)
+        return launch_behind(valid < SC::N ? fused_compress_kernel_capped<SC, LPB, true>
+                                           : fused_compress_kernel_capped<SC, LPB, false>,
+                             blocks, threads, smem, 1, st, in, out, n_lines, ld, valid, filt, tw);
+    else
+        return launch_behind(valid < SC::N ? fused_compress_kernel<SC, LPB, true>
+                                           : fused_compress_kernel<SC, LPB, false>,
+                             blocks, threads, smem, 1, st, in, out, n_lines, ld, valid, filt, tw);
 }
 
 template <class SC, int LPB>
@@ -97,11 +79,8 @@ cudaError_t launch_dft(const float2 *in, float2 *out, int64_t n_lines, int64_t l
     if (n_lines <= 0) return cudaSuccess;
     const int64_t blocks = (n_lines + LPB - 1) / LPB;
     constexpr int smem = smem_bytes_of<SC, LPB>();
-    if (inverse)
-        dft_lines_kernel<SC, LPB, true><<<(unsigned)blocks, SC::T * LPB, smem, st>>>(in, out, n_lines, ld, valid, tw);
-    else
-        dft_lines_kernel<SC, LPB, false><<<(unsigned)blocks, SC::T * LPB, smem, st>>>(in, out, n_lines, ld, valid, tw);
-    return cudaGetLastError();
+    return launch_behind(inverse ? dft_lines_kernel<SC, LPB, true> : dft_lines_kernel<SC, LPB, false>, blocks,
+                         SC::T * LPB, smem, 1, st, in, out, n_lines, ld, valid, tw);
 }
 
 // --- persistent schedules -----------------------------------------------
@@ -230,13 +209,13 @@ cudaError_t launch_streamed(const float2 *in, float2 *out, int64_t n_lines, int6
     if (n_lines <= 0) return cudaSuccess;
     if (valid < SC::N) return launch_fused<SC, 1>(in, out, n_lines, ld, valid, filt, tw, ctl, st);
     const int64_t blocks = (n_lines + LPB - 1) / LPB;
+    constexpr int threads = SC::T * LPB, smem = smem_bytes_of<SC, LPB>();
     if constexpr (SC::MINB > 0)
-        fused_streamed_kernel_capped<SC, LPB, ROLL><<<(unsigned)blocks, SC::T * LPB, smem_bytes_of<SC, LPB>(), st>>>(
-            in, out, n_lines, ld, filt, tw);
+        return launch_behind(fused_streamed_kernel_capped<SC, LPB, ROLL>, blocks, threads, smem, 1, st, in, out,
+                             n_lines, ld, filt, tw);
     else
-        fused_streamed_kernel<SC, LPB, ROLL><<<(unsigned)blocks, SC::T * LPB, smem_bytes_of<SC, LPB>(), st>>>(
-            in, out, n_lines, ld, filt, tw);
-    return cudaGetLastError();
+        return launch_behind(fused_streamed_kernel<SC, LPB, ROLL>, blocks, threads, smem, 1, st, in, out, n_lines, ld,
+                             filt, tw);
 }
 
 template <class SC, bool ROLL, int QL>
@@ -246,12 +225,11 @@ cudaError_t launch_range_ct(const float2 *in, float2 *img, int64_t n_lines, int6
     if (n_lines % QL) return cudaErrorInvalidValue;
     if constexpr (has_small_kernel<SC>()) {
         if (small_launch<SC>(n_lines))
-            return launch_behind(fused_range_ct_small_kernel<SC, QL>, (unsigned)(n_lines / QL), SC::T * QL,
-                                 ct_smem_bytes<SC, QL>(), st, in, img, ld_in, ld_img, filt, tw);
+            return launch_behind(fused_range_ct_small_kernel<SC, QL>, n_lines / QL, SC::T * QL,
+                                 ct_smem_bytes<SC, QL>(), 1, st, in, img, ld_in, ld_img, filt, tw);
     }
-    fused_range_ct_kernel<SC, QL, ROLL><<<(unsigned)(n_lines / QL), SC::T * QL, ct_smem_bytes<SC, QL>(), st>>>(
-        in, img, n_lines, ld_in, ld_img, filt, tw);
-    return cudaGetLastError();
+    return launch_behind(fused_range_ct_kernel<SC, QL, ROLL>, n_lines / QL, SC::T * QL, ct_smem_bytes<SC, QL>(), 1, st,
+                         in, img, n_lines, ld_in, ld_img, filt, tw);
 }
 
 template <class SC, int QC, bool ROLL>
@@ -259,25 +237,15 @@ cudaError_t launch_range_ct_cluster(const float2 *in, float2 *img, int64_t n_lin
                                     const float2 *filt, const float2 *tw, cudaStream_t st) {
     if (n_lines <= 0) return cudaSuccess;
     if (n_lines % QC) return cudaErrorInvalidValue;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)n_lines, 1, 1);
-    cfg.blockDim = dim3(SC::T, 1, 1);
-    cfg.dynamicSmemBytes = smem_bytes_of<SC, 1>();
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = QC;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    constexpr int smem = smem_bytes_of<SC, 1>();
     if constexpr (ct_tma_ok<SC, QC, ROLL>()) {
         CUtensorMap m;
         if (image_tensor_map(&m, img, n_lines, SC::N, ld_img, 1, 256))
-            return cudaLaunchKernelEx(&cfg, fused_range_ct_tma_kernel<SC, QC, ROLL>, in, img, m, ld_in, ld_img, filt,
-                                      tw);
+            return launch_behind(fused_range_ct_tma_kernel<SC, QC, ROLL>, n_lines, SC::T, smem, QC, st, in, img, m,
+                                 ld_in, ld_img, filt, tw);
     }
-    return cudaLaunchKernelEx(&cfg, fused_range_ct_cluster_kernel<SC, QC, ROLL>, in, img, ld_in, ld_img, filt, tw);
+    return launch_behind(fused_range_ct_cluster_kernel<SC, QC, ROLL>, n_lines, SC::T, smem, QC, st, in, img, ld_in,
+                         ld_img, filt, tw);
 }
 
 template <class SC, int LPB, bool ROLL>

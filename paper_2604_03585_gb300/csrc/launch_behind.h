@@ -1,0 +1,42 @@
+// Launching a kernel programmatically behind the last one on its stream.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace sar {
+
+// Up to this many threads in all, about two waves of the GPU, the time from
+// one kernel's end to the next one's first instruction counts: it is then
+// launched while its predecessor still runs and waits for it in the kernel
+// (sar_common.cuh: grid_enter, which every kernel launched here begins with).
+// Above, blocks that wait would only keep SMs from other streams' kernels.
+constexpr int64_t kBehindThreads = 2 * 152 * 2048;
+
+// cluster: blocks per thread-block cluster (1: none).
+template <class... Params, class... Args>
+cudaError_t launch_behind(void (*kernel)(Params...), int64_t blocks, int threads, int smem, int cluster,
+                          cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks, 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)cluster;
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
+    if (blocks * threads <= kBehindThreads) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = (unsigned)n;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+}  // namespace sar

@@ -297,6 +297,7 @@ template <class SC, int LPB, bool RAGGED>
 __device__ __forceinline__ void fused_compress_body(const float2* in, float2* out, int64_t n_lines, int64_t ld,
                                                     int valid, const float2* filt, const float2* tw) {
     extern __shared__ float2 smem_dyn[];
+    grid_enter();
     const int lib = threadIdx.x / SC::T;
     const int t = threadIdx.x % SC::T;
     const int64_t line = (int64_t)blockIdx.x * LPB + lib;
@@ -336,9 +337,6 @@ fused_compress_kernel_capped(const float2* in, float2* out, int64_t n_lines, int
 // lines spread over the SMs.  Same arithmetic as the kernels above:
 // bit-identical.  Two passes of a 256 x 256 scene: 11.9 -> 9.6 us a scene, back
 // to back from Python (which then is busy for 9.4 us of them).
-__device__ __forceinline__ void grid_release_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
-__device__ __forceinline__ void grid_wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 template <class SC>
 struct SmallTables {
     static_assert(SC::P == 2, "two-pass lengths");
@@ -423,6 +421,7 @@ __global__ void __launch_bounds__(SC::T * LPB, min_blocks_128<SC, LPB>())
 dft_lines_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld,
                  int valid, const float2* tw) {
     extern __shared__ float2 smem_dyn[];
+    grid_enter();
     const int lib = threadIdx.x / SC::T;
     const int t = threadIdx.x % SC::T;
     const int64_t line = (int64_t)blockIdx.x * LPB + lib;

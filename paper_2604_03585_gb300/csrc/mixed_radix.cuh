@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(kMixedThreads, MINB)
 fused_mixed_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, const float2* filt, const float2* tw,
                    MixedGeom geo) {
     extern __shared__ float2 smem_mixed[];
+    grid_enter();
     const int T = geo.T, lib = threadIdx.x / T, t = threadIdx.x % T;
     const int64_t line = (int64_t)blockIdx.x * (kMixedThreads / T) + lib;
     const bool live = line < n_lines;
@@ -305,6 +306,7 @@ fused_mixed3_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, 
     constexpr uint32_t MA = split_magic(SA), MB = split_magic(SB);
     constexpr int LPB = kMixedThreads / T, PADN = mixed3_smem<N, T, PADDIV>() / LPB / (int)sizeof(float2);
     extern __shared__ float2 smem_mixed[];
+    grid_enter();
     const int lib = threadIdx.x / T, t = threadIdx.x % T;
     const int64_t line = (int64_t)blockIdx.x * LPB + lib;
     const bool live = line < n_lines;
@@ -426,6 +428,7 @@ __device__ __forceinline__ void fused_mixed3_ct_body(const float2* in, float2* i
     constexpr int NQ = N / QC, RS = NQ + 4, GA = (SA + T - 1) / T;
     static_assert(N % QC == 0 && 4 * RS <= LPB * PADN, "four receive rows fit the block's line buffers");
     extern __shared__ float2 smem_mixed[];
+    grid_enter();
     const int lib = threadIdx.x / T, t = threadIdx.x % T;
     int rank = 0;
     if constexpr (QC > 1) rank = (int)cg::this_cluster().block_rank();
@@ -550,9 +553,8 @@ fused_mixed3_ct_tma_kernel(const float2* in, float2* img, const __grid_constant_
 template <int MINB>
 cudaError_t launch_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, const float2* filt,
                           const float2* tw, const MixedGeom& g, int lines_per_block, int smem, cudaStream_t st) {
-    fused_mixed_kernel<MINB><<<(unsigned)((n_lines + lines_per_block - 1) / lines_per_block), kMixedThreads, smem,
-                               st>>>(in, out, n_lines, ld, filt, tw, g);
-    return cudaGetLastError();
+    return launch_behind(fused_mixed_kernel<MINB>, (n_lines + lines_per_block - 1) / lines_per_block, kMixedThreads,
+                         smem, 1, st, in, out, n_lines, ld, filt, tw, g);
 }
 template <int MINB>
 cudaError_t set_smem(int bytes) {

@@ -13,9 +13,8 @@ cudaError_t launch3(const float2* in, float2* out, int64_t n_lines, int64_t ld, 
                     int, cudaStream_t st) {
     constexpr int LPB = kMixedThreads / T, smem = mixed3_smem<N, T, PD>();
     static_assert(smem <= kMixedSmemMax, "within the shared memory the kernel is set up for");
-    fused_mixed3_kernel<N, RA, RB, RC, T, MINB, PD>
-        <<<(unsigned)((n_lines + LPB - 1) / LPB), kMixedThreads, smem, st>>>(in, out, n_lines, ld, filt, tw);
-    return cudaGetLastError();
+    return launch_behind(fused_mixed3_kernel<N, RA, RB, RC, T, MINB, PD>, (n_lines + LPB - 1) / LPB, kMixedThreads,
+                         smem, 1, st, in, out, n_lines, ld, filt, tw);
 }
 template <int N, int RA, int RB, int RC, int T, int MINB, int PD>
 cudaError_t launch3_dft(const float2* in, float2* out, int64_t n_lines, int64_t ld, int valid, const float2* tw,
@@ -33,25 +32,14 @@ cudaError_t launch3_ct(const float2* in, float2* img, int64_t n_lines, int64_t l
     constexpr int LPB = kMixedThreads / T, QC = 4 / LPB;
     if (n_lines <= 0) return cudaSuccess;
     if (n_lines % 4 || ld_img % 2) return cudaErrorInvalidValue;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(n_lines / LPB), 1, 1);
-    cfg.blockDim = dim3(kMixedThreads, 1, 1);
-    cfg.dynamicSmemBytes = mixed3_smem<N, T, PD>();
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = QC;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = QC > 1 ? 1 : 0;
+    constexpr int smem = mixed3_smem<N, T, PD>();
     using G = MixedCtGeom<N, T, PD>;
     CUtensorMap m;
     if (image_tensor_map(&m, img, n_lines, N, ld_img, QC, G::BR))
-        return cudaLaunchKernelEx(&cfg, fused_mixed3_ct_tma_kernel<N, RA, RB, RC, T, MINB, PD>, in, img, m, ld_in,
-                                  ld_img, filt, tw);
-    return cudaLaunchKernelEx(&cfg, fused_mixed3_ct_kernel<N, RA, RB, RC, T, MINB, PD>, in, img, ld_in, ld_img, filt,
-                              tw);
+        return launch_behind(fused_mixed3_ct_tma_kernel<N, RA, RB, RC, T, MINB, PD>, n_lines / LPB, kMixedThreads,
+                             smem, QC, st, in, img, m, ld_in, ld_img, filt, tw);
+    return launch_behind(fused_mixed3_ct_kernel<N, RA, RB, RC, T, MINB, PD>, n_lines / LPB, kMixedThreads, smem, QC, st,
+                         in, img, ld_in, ld_img, filt, tw);
 }
 template <int N, int RA, int RB, int RC, int T, int MINB, int PD>
 cudaError_t attr3() {

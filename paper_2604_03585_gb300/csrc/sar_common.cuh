@@ -14,6 +14,20 @@
 namespace sar {
 
 // ---------------------------------------------------------------------------
+// programmatic launches (launch_behind.h)
+// ---------------------------------------------------------------------------
+// Lets the stream's next kernel be launched, and waits until the one before is
+// complete and its memory visible; both return at once in an ordinary launch.
+// Data that a predecessor may have written must not be read as read-only
+// (ld.global.nc): the predecessor can still run when this grid starts.
+__device__ __forceinline__ void grid_release_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void grid_wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_enter() {
+    grid_release_dependents();
+    grid_wait_predecessor();
+}
+
+// ---------------------------------------------------------------------------
 // complex float helpers (float2 = interleaved complex64)
 // ---------------------------------------------------------------------------
 // Complex add and subtract as one packed two-wide FP32 instruction each

@@ -160,6 +160,7 @@ template <class SC, int LPB, bool ROLL>
 __device__ __forceinline__ void fused_streamed_body(const float2* in, float2* out, int64_t n_lines, int64_t ld,
                                                     const float2* filt, const float2* tw) {
     extern __shared__ float2 smem_dyn[];
+    grid_enter();
     const int lib = threadIdx.x / SC::T;
     const int t = threadIdx.x % SC::T;
     const int64_t line = (int64_t)blockIdx.x * LPB + lib;
@@ -269,6 +270,7 @@ template <class SC, int QL, bool ROLL>
 __device__ __forceinline__ void fused_range_ct_body(const float2* in, float2* img, int64_t n_lines, int64_t ld_in,
                                                     int64_t ld_img, const float2* filt, const float2* tw) {
     extern __shared__ float2 smem_dyn[];
+    grid_enter();
     const int lib = threadIdx.x / SC::T;
     const int t = threadIdx.x % SC::T;
     const int64_t a0 = (int64_t)blockIdx.x * QL;
@@ -351,6 +353,7 @@ __device__ __forceinline__ void fused_range_ct_cluster_body(const float2* in, fl
                                                             const float2* tw, const CUtensorMap* tmap = nullptr) {
     namespace cg = cooperative_groups;
     extern __shared__ float2 smem_dyn[];
+    grid_enter();
     cg::cluster_group cluster = cg::this_cluster();
     const int t = threadIdx.x;
     const int rank = (int)cluster.block_rank();

@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(SC::T * LPB, min_blocks_128<SC, LPB>())
 fused_wrap_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, int n, const float2* filt,
                   const float2* tw) {
     extern __shared__ float2 smem_dyn[];
+    grid_enter();
     const int lib = threadIdx.x / SC::T;
     const int t = threadIdx.x % SC::T;
     const int64_t line = (int64_t)blockIdx.x * LPB + lib;
@@ -126,9 +127,8 @@ cudaError_t launch_wrap(const float2* in, float2* out, int64_t n_lines, int64_t 
     if (n_lines <= 0) return cudaSuccess;
     if (valid < 1 || 2 * (int64_t)valid - 1 > SC::N || ld < valid) return cudaErrorInvalidValue;
     const int64_t blocks = (n_lines + LPB - 1) / LPB;
-    fused_wrap_kernel<SC, LPB, ROLL><<<(unsigned)blocks, SC::T * LPB, smem_bytes_of<SC, LPB>(), st>>>(
-        in, out, n_lines, ld, valid, filt, tw);
-    return cudaGetLastError();
+    return launch_behind(fused_wrap_kernel<SC, LPB, ROLL>, blocks, SC::T * LPB, smem_bytes_of<SC, LPB>(), 1, st, in,
+                         out, n_lines, ld, valid, filt, tw);
 }
 
 template <class SC, int LPB, bool ROLL>
