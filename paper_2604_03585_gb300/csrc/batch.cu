@@ -222,12 +222,13 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, sar_
     }
     // how the range items of each length run.  Long lines are stored in sets of
     // four, all but the last parked in the scratch (none if there is no memory
-    // for it: then an item is the lines its worker holds at once).  Where that
-    // would leave workers idle, the whole block takes as many lines as it holds
-    // and parks none: below two sets for each worker of 128 threads at 2048 and
-    // 4096 samples (one strip of 4096 x 400: 37 us against 90), below one set
-    // for each block at 8192 (8192 x 300: 53 us against 108; x 1000: 178
-    // against 157) and 16384 (x 300: 110 against 137; x 1000: 352 against 307)
+    // for it: then an item is the lines its worker holds at once).  A few waves
+    // of such sets leave workers idle at the end: there the whole block takes
+    // as many lines as it holds and parks none.  One strip, us against us with
+    // sets: 4096 x 400 37 / 90, 4096 x 5000 466 / 526 (limit: four sets for
+    // each worker of 128 threads); 8192 x 300 53 / 108, x 1570 275 / 318, x 2400
+    // 486 / 427 (three per block); 16384 x 300 110 / 137, x 700 237 / 286, x
+    // 1500 580 / 543 (two per block)
     const int64_t blocks = sar::batch_grid(), workers = blocks * (sar::kBatchThreads / 128);
     int64_t sets_short = 0, sets_8192 = 0, sets_16384 = 0, sets_tiny = 0;
     for (int32_t i = 0; i < count; ++i) {
@@ -238,7 +239,7 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, sar_
         else if (strips[i].n_range <= 512) sets_tiny += (strips[i].n_az + 7) / 8;
     }
     auto few = [&](int64_t n) {
-        return n == 16384 ? sets_16384 < blocks : n == 8192 ? sets_8192 < blocks : sets_short < 2 * workers;
+        return n == 16384 ? sets_16384 < 2 * blocks : n == 8192 ? sets_8192 < 3 * blocks : sets_short < 4 * workers;
     };
     auto range_geometry = [&](int64_t n) {
         sar::BatchGeom g = sar::batch_geometry((int)n, few(n));

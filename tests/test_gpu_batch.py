@@ -142,7 +142,7 @@ def test_one_launch_equals_multi_kernel_graph(sar):
 @pytest.mark.parametrize("shapes", [
     # azimuth lengths 512 ... 4096 side by side in the workers of a block, several lines per worker item,
     # range items of 8192 and 16384 samples in two and four rounds with a remainder
-    [(4096, 2101), (4096, 1025), (8192, 613), (16384, 614), (2048, 1026), (4096, 2049)],
+    [(4096, 4101), (4096, 3001), (8192, 1830), (16384, 1222), (2048, 1026), (4096, 2049)],
     # azimuth lines of the whole block (8192, 16384) beside short ones, few items
     [(256, 4097), (512, 9000), (8192, 3), (16384, 5), (16384, 1), (1024, 257)],
     # several sets of short range lines per item, with a remainder
