@@ -56,15 +56,20 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // Step 1: C-point DFTs over n1 and the twiddle W_N^{n2 k1}, pushed to block
 // k1 at position n2 (PADDED: at the line engine's padded shared-memory slot of
 // n2), one n2 at a time (C values live).  roots[k1 M + n2] = W_N^{k1 n2}
-// (one contiguous row per k1).  The block announces itself on the cluster barrier at once and waits
-// for the others just before its first remote store.
+// (one contiguous row per k1).  The block announces itself on the cluster
+// barrier at once and waits for the others just before its first remote store.
+// Streamed, four n2 of up to 8 values are in flight, one of 16 (65536 points
+// as 8 x 8192, 512 lines: 290.8 us against 292.0 with two; 131072 as 16 x
+// 8192, 256 lines: 375.4 against 389.0).  Staggered starts (line_engine.cuh)
+// gain nothing here, where cluster barriers keep the blocks in step: 290.1
+// without against 292.0.
 template <class SC, int C, bool RAGGED, bool CONJ_IN, bool PADDED = false>
 __device__ __forceinline__ void cluster_first_stage(const float2* src, int valid, const float2* roots, int t,
                                                     int rank, float2* sm,
                                                     cooperative_groups::cluster_group& cluster) {
     using G = ClusterGeom<SC, C>;
     cluster_arrive_relaxed();
-#pragma unroll(PADDED ? 2 : G::EQ)
+#pragma unroll(PADDED ? (C < 16 ? 4 : 1) : G::EQ)
     for (int i = 0; i < G::EQ; ++i) {
         const int n2 = rank * G::Q + t + SC::T * i;
         float2 a[C];
@@ -181,7 +186,7 @@ cluster_streamed_kernel(const float2* in, float2* out, int64_t ld, const float2*
     __syncthreads();
     const float2* tw2 = tw + R1 * S1;
     if constexpr (SC::P == 3) {
-        streamed_mid_pass<SC, 1, SC::R2, SC::S2, false, ROLL, true>(sm, tw2, t, 0);
+        streamed_mid_pass<SC, 1, SC::R2, SC::S2, false, ROLL>(sm, tw2, t, 0);
         sub_sync<SC, 1>(0);
     }
     // last forward pass, this block's filter slice, first inverse pass
@@ -196,7 +201,9 @@ cluster_streamed_kernel(const float2* in, float2* out, int64_t ld, const float2*
     for (int s = 0; s < G1; ++s) {
         const int lo = t + SC::T * s;
         float2 x[R1];
-        streamed_final_group<SC, 1>(sm, tw, t, 0, s, x);
+        grp_smem_load<R1, S1>(sm, lo, SC::PADSH, x);
+        grp_twiddle<R1, S1, true>(tw, lo, x);
+        dft_reg<R1, true>(x);
 #pragma unroll
         for (int r = 0; r < R1; ++r) x[r] = cmulc(x[r], roots[rank * G::M + lo + r * S1]);
         grp_smem_store<R1, S1>(sm, lo, SC::PADSH, x);
@@ -213,7 +220,12 @@ cluster_streamed_kernel(const float2* in, float2* out, int64_t ld, const float2*
 #pragma unroll
         for (int n1 = 0; n1 < C; ++n1) __stcs(dst + n1 * G::M + n2, b[n1]);
     }
-    cluster.sync();   // keep this block's shared memory until every block has pulled
+    // keep this block's shared memory until every block has pulled: the pulled
+    // values are stored above, so nothing is left to order, and a releasing
+    // arrive would wait for those stores (32768 / 65536 / 131072 points, 2^25
+    // samples: 244.7 / 289.2 / 377.6 us with it, 237.5 / 281.1 / 361.0 without)
+    cluster_arrive_relaxed();
+    cluster_wait();
 }
 
 // Stand-alone FFT of a line, natural-order output (unnormalised; the inverse
