@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(kTile * kRowsPerPass)
 corner_turn_kernel(const float2 *in, float2 *__restrict__ out, int64_t rows, int64_t cols,
                    int64_t tiles_c) {
     __shared__ float2 tile[kTile][kTile + 1];
-    grid_enter();
+    grid_wait_predecessor();
     const int64_t tr = blockIdx.x / tiles_c;           // tile row (over `rows`)
     const int64_t tc = blockIdx.x % tiles_c;           // tile column (over `cols`)
     const int tx = threadIdx.x % kTile, ty = threadIdx.x / kTile;
@@ -34,6 +34,7 @@ corner_turn_kernel(const float2 *in, float2 *__restrict__ out, int64_t rows, int
         if (full || (r < rows && c < cols)) tile[ty + j][tx] = in[r * cols + c];
     }
     __syncthreads();
+    grid_release_dependents();
 #pragma unroll
     for (int j = 0; j < kTile; j += kRowsPerPass) {
         const int64_t c = c0 + ty + j, r = r0 + tx;       // destination row c, column r
@@ -56,7 +57,7 @@ __global__ void __launch_bounds__(256)
 corner_turn64_kernel(const float4 *in, float4 *__restrict__ out, int64_t rows, int64_t cols,
                      int64_t tiles_c) {
     __shared__ float4 tile[kBig * 32];                 // 64 rows x 32 chunks of 16 B
-    grid_enter();
+    grid_wait_predecessor();
     const int64_t tr = blockIdx.x / tiles_c, tc = blockIdx.x % tiles_c;
     const int64_t r0 = tr * kBig, c0 = tc * kBig;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -68,6 +69,7 @@ corner_turn64_kernel(const float4 *in, float4 *__restrict__ out, int64_t rows, i
         tile[ct_chunk(r, lane)] = in[(r0 + r) * cols2 + c0 / 2 + lane];
     }
     __syncthreads();
+    grid_release_dependents();
     // store: warp w writes output rows c = 2*(w + 8k) and c + 1; lane l covers
     // input rows 2l and 2l + 1 of the tile
 #pragma unroll

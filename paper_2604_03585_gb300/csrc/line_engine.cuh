@@ -297,7 +297,7 @@ template <class SC, int LPB, bool RAGGED>
 __device__ __forceinline__ void fused_compress_body(const float2* in, float2* out, int64_t n_lines, int64_t ld,
                                                     int valid, const float2* filt, const float2* tw) {
     extern __shared__ float2 smem_dyn[];
-    grid_enter();
+    grid_wait_predecessor();
     const int lib = threadIdx.x / SC::T;
     const int t = threadIdx.x % SC::T;
     const int64_t line = (int64_t)blockIdx.x * LPB + lib;
@@ -308,6 +308,7 @@ __device__ __forceinline__ void fused_compress_body(const float2* in, float2* ou
     forward_passes<SC, LPB>(v, sm, tw, t, lib);
     filter_multiply<SC>(filt, t, v);
     inverse_passes<SC, LPB>(v, sm, tw, t, lib);
+    grid_release_dependents();
     global_store<SC, RAGGED>(out + line * ld, valid, t, v);
 }
 
@@ -335,8 +336,8 @@ fused_compress_kernel_capped(const float2* in, float2* out, int64_t n_lines, int
 // it drains, and only then wait for it (griddepcontrol.wait: complete, its
 // memory visible) and touch the caller's data.  One warp per block, so that the
 // lines spread over the SMs.  Same arithmetic as the kernels above:
-// bit-identical.  Two passes of a 256 x 256 scene: 11.9 -> 9.6 us a scene, back
-// to back from Python (which then is busy for 9.4 us of them).
+// bit-identical.  256 lines of 256, 512, 1024 samples back to back: 3.1, 4.3,
+// 4.4 -> 2.7, 4.0, 4.1 us, folded 3.2, 4.6, 5.8 -> 2.0, 3.2, 3.9 us.
 template <class SC>
 struct SmallTables {
     static_assert(SC::P == 2, "two-pass lengths");
@@ -385,7 +386,6 @@ __global__ void __launch_bounds__(SC::T* small_lines_per_block<SC>())
 fused_small_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, const float2* filt, const float2* tw) {
     constexpr int LPB = small_lines_per_block<SC>();
     extern __shared__ float2 smem_dyn[];
-    grid_release_dependents();
     const int lib = threadIdx.x / SC::T, t = threadIdx.x % SC::T;
     const int64_t line = (int64_t)blockIdx.x * LPB + lib;
     if (line >= n_lines) return;
@@ -395,6 +395,7 @@ fused_small_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, c
     float2 v[SC::E];
     global_load<SC, false>(in + line * ld, SC::N, t, v);
     small_compress<SC, LPB>(v, tab, smem_dyn + lib * SC::SMEM_ELEMS, t, lib);
+    grid_release_dependents();
     global_store<SC, false>(out + line * ld, SC::N, t, v);
 }
 
@@ -421,7 +422,7 @@ __global__ void __launch_bounds__(SC::T * LPB, min_blocks_128<SC, LPB>())
 dft_lines_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld,
                  int valid, const float2* tw) {
     extern __shared__ float2 smem_dyn[];
-    grid_enter();
+    grid_wait_predecessor();
     const int lib = threadIdx.x / SC::T;
     const int t = threadIdx.x % SC::T;
     const int64_t line = (int64_t)blockIdx.x * LPB + lib;
@@ -448,6 +449,7 @@ dft_lines_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld,
         }
     }
     line_sync<SC, LPB>(lib);
+    grid_release_dependents();
     float2* dst = out + line * SC::N;  // outputs are dense lines of N
 #pragma unroll
     for (int j = 0; j < SC::E; ++j) {

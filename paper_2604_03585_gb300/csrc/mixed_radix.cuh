@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kMixedThreads, MINB)
 fused_mixed_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, const float2* filt, const float2* tw,
                    MixedGeom geo) {
     extern __shared__ float2 smem_mixed[];
-    grid_enter();
+    grid_wait_predecessor();
     const int T = geo.T, lib = threadIdx.x / T, t = threadIdx.x % T;
     const int64_t line = (int64_t)blockIdx.x * (kMixedThreads / T) + lib;
     const bool live = line < n_lines;
@@ -278,6 +278,7 @@ fused_mixed_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, c
         if (live) mpass<kInvMid, false>(geo.R[i], geo.S[i], geo.M[i], n, t, T, src, dst, sm, tw + geo.tw_off[i], filt);
         __syncthreads();
     }
+    grid_release_dependents();
     if (live) mpass<kInvFirst, false>(geo.R[0], geo.S[0], geo.M[0], n, t, T, src, dst, sm, tw + geo.tw_off[0], filt);
 }
 
@@ -306,7 +307,7 @@ fused_mixed3_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, 
     constexpr uint32_t MA = split_magic(SA), MB = split_magic(SB);
     constexpr int LPB = kMixedThreads / T, PADN = mixed3_smem<N, T, PADDIV>() / LPB / (int)sizeof(float2);
     extern __shared__ float2 smem_mixed[];
-    grid_enter();
+    grid_wait_predecessor();
     const int lib = threadIdx.x / T, t = threadIdx.x % T;
     const int64_t line = (int64_t)blockIdx.x * LPB + lib;
     const bool live = line < n_lines;
@@ -330,6 +331,7 @@ fused_mixed3_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, 
         for (int g = t; g < N / RB; g += T)
             mgroup<RB, kInvMid, false, PADDIV>(g, SB, MB, N / RB, src, dst, sm, twb, filt);
     __syncthreads();
+    grid_release_dependents();
     if (live)
         for (int g = t; g < N / RA; g += T)
             mgroup<RA, kInvFirst, false, PADDIV>(g, SA, MA, N / RA, src, dst, sm, tw, filt);
@@ -428,7 +430,7 @@ __device__ __forceinline__ void fused_mixed3_ct_body(const float2* in, float2* i
     constexpr int NQ = N / QC, RS = NQ + 4, GA = (SA + T - 1) / T;
     static_assert(N % QC == 0 && 4 * RS <= LPB * PADN, "four receive rows fit the block's line buffers");
     extern __shared__ float2 smem_mixed[];
-    grid_enter();
+    grid_wait_predecessor();
     const int lib = threadIdx.x / T, t = threadIdx.x % T;
     int rank = 0;
     if constexpr (QC > 1) rank = (int)cg::this_cluster().block_rank();
@@ -481,6 +483,7 @@ __device__ __forceinline__ void fused_mixed3_ct_body(const float2* in, float2* i
         cg::this_cluster().sync();   // the pushes have landed; only local reads from here on
     else
         __syncthreads();
+    grid_release_dependents();
     if constexpr (TMA) {
         // the receive rows rewritten bin-major in place (bin j's four samples
         // at stg[2j], stg[2j + 1]) and stored as NB boxes of the block's plane

@@ -16,16 +16,16 @@ namespace sar {
 // ---------------------------------------------------------------------------
 // programmatic launches (launch_behind.h)
 // ---------------------------------------------------------------------------
-// Lets the stream's next kernel be launched, and waits until the one before is
-// complete and its memory visible; both return at once in an ordinary launch.
-// Data that a predecessor may have written must not be read as read-only
-// (ld.global.nc): the predecessor can still run when this grid starts.
+// A kernel waits until the one before it on the stream is complete and its
+// memory visible, and lets the next one be launched; both return at once in an
+// ordinary launch.  Data that a predecessor may have written must not be read
+// as read-only (ld.global.nc): the predecessor can still run when this grid
+// starts.  The release comes late, when a block has only its stores left:
+// released at the start, the next grid's blocks are handed out while this one's
+// still fill some SMs, and stay unevenly spread (800 lines of 1024, folded, back
+// to back: 15.4 us against 8.2 in ordinary launches).
 __device__ __forceinline__ void grid_release_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void grid_wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_enter() {
-    grid_release_dependents();
-    grid_wait_predecessor();
-}
 
 // ---------------------------------------------------------------------------
 // complex float helpers (float2 = interleaved complex64)

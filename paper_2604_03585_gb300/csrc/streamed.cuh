@@ -160,7 +160,7 @@ template <class SC, int LPB, bool ROLL>
 __device__ __forceinline__ void fused_streamed_body(const float2* in, float2* out, int64_t n_lines, int64_t ld,
                                                     const float2* filt, const float2* tw) {
     extern __shared__ float2 smem_dyn[];
-    grid_enter();
+    grid_wait_predecessor();
     const int lib = threadIdx.x / SC::T;
     const int t = threadIdx.x % SC::T;
     const int64_t line = (int64_t)blockIdx.x * LPB + lib;
@@ -169,6 +169,7 @@ __device__ __forceinline__ void fused_streamed_body(const float2* in, float2* ou
     float2* dst = out + line * ld;
     constexpr int R1 = SC::R1, S1 = SC::S1, G1 = SC::E / R1;
     streamed_until_last<SC, LPB, ROLL>(in + line * ld, sm, filt, tw, t, lib);
+    grid_release_dependents();
     // ---- inverse pass 1: shared memory -> twiddle -> inverse DFT -> HBM
 #pragma unroll(ROLL ? 1 : G1)
     for (int s = 0; s < G1; ++s) {
@@ -270,7 +271,7 @@ template <class SC, int QL, bool ROLL>
 __device__ __forceinline__ void fused_range_ct_body(const float2* in, float2* img, int64_t n_lines, int64_t ld_in,
                                                     int64_t ld_img, const float2* filt, const float2* tw) {
     extern __shared__ float2 smem_dyn[];
-    grid_enter();
+    grid_wait_predecessor();
     const int lib = threadIdx.x / SC::T;
     const int t = threadIdx.x % SC::T;
     const int64_t a0 = (int64_t)blockIdx.x * QL;
@@ -287,6 +288,7 @@ __device__ __forceinline__ void fused_range_ct_body(const float2* in, float2* im
 #pragma unroll
         for (int r = 0; r < R1; ++r) v[s * R1 + r] = x[r];
     }
+    grid_release_dependents();
     store_corner_turned<SC, QL>(v, smem_dyn, t, lib, img, ld_img, a0);
 }
 
@@ -296,7 +298,6 @@ __global__ void __launch_bounds__(SC::T* QL)
 fused_range_ct_small_kernel(const float2* in, float2* img, int64_t ld_in, int64_t ld_img, const float2* filt,
                             const float2* tw) {
     extern __shared__ float2 smem_dyn[];
-    grid_release_dependents();
     const int lib = threadIdx.x / SC::T, t = threadIdx.x % SC::T;
     const int64_t a0 = (int64_t)blockIdx.x * QL;
     SmallTables<SC> tab;
@@ -305,6 +306,7 @@ fused_range_ct_small_kernel(const float2* in, float2* img, int64_t ld_in, int64_
     float2 v[SC::E];
     global_load<SC, false>(in + (a0 + lib) * ld_in, SC::N, t, v);
     small_compress<SC, QL>(v, tab, smem_dyn + lib * SC::SMEM_ELEMS, t, lib);
+    grid_release_dependents();
     store_corner_turned<SC, QL>(v, smem_dyn, t, lib, img, ld_img, a0);
 }
 
@@ -353,7 +355,7 @@ __device__ __forceinline__ void fused_range_ct_cluster_body(const float2* in, fl
                                                             const float2* tw, const CUtensorMap* tmap = nullptr) {
     namespace cg = cooperative_groups;
     extern __shared__ float2 smem_dyn[];
-    grid_enter();
+    grid_wait_predecessor();
     cg::cluster_group cluster = cg::this_cluster();
     const int t = threadIdx.x;
     const int rank = (int)cluster.block_rank();
@@ -392,6 +394,7 @@ __device__ __forceinline__ void fused_range_ct_cluster_body(const float2* in, fl
         }
     }
     cluster.sync();
+    grid_release_dependents();
     if constexpr (TMA) {
         static_assert(ct_tma_ok<SC, QC, ROLL>(), "four lines, whole boxes of 256 bins");
         constexpr int NIT = NQ * 2 / SC::T;

@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(SC::T * LPB, min_blocks_128<SC, LPB>())
 fused_wrap_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, int n, const float2* filt,
                   const float2* tw) {
     extern __shared__ float2 smem_dyn[];
-    grid_enter();
+    grid_wait_predecessor();
     const int lib = threadIdx.x / SC::T;
     const int t = threadIdx.x % SC::T;
     const int64_t line = (int64_t)blockIdx.x * LPB + lib;
@@ -42,6 +42,7 @@ fused_wrap_kernel(const float2* in, float2* out, int64_t n_lines, int64_t ld, in
         grp_smem_store<R1, S1>(sm, lo, SC::PADSH, x);
     }
     line_sync<SC, LPB>(lib);
+    grid_release_dependents();
     // y[m] = z[m] + z[m + n], m + n <= 2n - 1 < L
     float2* dst = out + line * ld;
     for (int m = t; m < n; m += SC::T) {
