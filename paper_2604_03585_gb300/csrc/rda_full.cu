@@ -19,6 +19,7 @@
 // range bin n never enters a rounded sum (at n ~ 8000 the FP32 spacing is
 // 1e-3 samples, which would cost ~1e-3 relative error on a half-band signal).
 #include "../../include/sar.h"
+#include "launch_behind.h"
 #include "streamed.cuh"
 #include "registry.h"
 #include "tables.h"
@@ -160,12 +161,15 @@ __device__ __forceinline__ void rc_interp(const float (&frac)[kRcWide], float2 (
 }
 
 __global__ void __launch_bounds__(kRcCols * kRcWarps)
-rcmc_tile_kernel(const float2* __restrict__ in, float2* __restrict__ out, int n_range, int n_f,
+rcmc_tile_kernel(const float2* in, float2* __restrict__ out, int n_range, int n_f,
                  const RdColumn* __restrict__ cols, float rn_hi, float rn_lo, int staged_rows) {
     extern __shared__ float2 tile[];   // [staged_rows][32]
+    grid_wait_predecessor();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int j = blockIdx.x * kRcCols + lane;
-    const int n0 = blockIdx.y * kRcRows;
+    // tiles of one range of bins are neighbours, as their rows are
+    const int tiles_f = (n_f + kRcCols - 1) / kRcCols;
+    const int j = (int)(blockIdx.x % tiles_f) * kRcCols + lane;
+    const int n0 = (int)(blockIdx.x / tiles_f) * kRcRows;
     const int n1 = min(n0 + kRcRows, n_range) - 1;
     const bool jok = j < n_f;
     const RdColumn c = cols[jok ? j : n_f - 1];
@@ -240,6 +244,7 @@ __global__ void __launch_bounds__(SC::T, SC::T >= 256 ? min_blocks_128<SC, 1>() 
 az_streamed_kernel(const float2* in, float2* out, int64_t n_lines, const float2* tw, const RdColumn* cols,
                    double r_near) {
     extern __shared__ float2 smem_dyn[];
+    grid_wait_predecessor();
     const int t = threadIdx.x;
     const int64_t line = blockIdx.x;
     if (line >= n_lines) return;
@@ -307,6 +312,7 @@ az_streamed_kernel(const float2* in, float2* out, int64_t n_lines, const float2*
         for (int r = 0; r < RL; ++r) sm[smem_pos(natural_index<SC>(pass_group<SC, RL, 1>(t, s), r), SC::PADSH)] = v[s * RL + r];
     }
     __syncthreads();
+    grid_release_dependents();
     constexpr float inv_n = 1.0f / SC::N;
     float2* dst = out + line * SC::N;
 #pragma unroll
@@ -335,8 +341,8 @@ cudaError_t launch_az(const float2* in, float2* out, int64_t n_lines, const floa
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    az_streamed_kernel<SC, COMPRESS><<<(unsigned)n_lines, SC::T, smem, st>>>(in, out, n_lines, tw, cols, r_near);
-    return cudaGetLastError();
+    return launch_behind(az_streamed_kernel<SC, COMPRESS>, n_lines, SC::T, smem, 1, st, in, out, n_lines, tw, cols,
+                         r_near);
 }
 
 template <bool COMPRESS>
@@ -392,10 +398,9 @@ cudaError_t launch_rcmc(int taps, const float2* in, float2* out, int n_range, in
         if (e != cudaSuccess) return e;
     }
     const float rn_hi = (float)r_near, rn_lo = (float)(r_near - (double)rn_hi);
-    const dim3 grid((unsigned)((n_f + kRcCols - 1) / kRcCols), (unsigned)((n_range + kRcRows - 1) / kRcRows));
-    rcmc_tile_kernel<<<grid, kRcCols * kRcWarps, smem, st>>>(in, out, n_range, n_f, (const RdColumn*)cols, rn_hi,
-                                                            rn_lo, staged_rows);
-    return cudaGetLastError();
+    const int tiles_f = (n_f + kRcCols - 1) / kRcCols, tiles_r = (n_range + kRcRows - 1) / kRcRows;
+    return launch_behind(rcmc_tile_kernel, (int64_t)tiles_f * tiles_r, kRcCols * kRcWarps, (int)smem, 1, st, in, out,
+                         n_range, n_f, (const RdColumn*)cols, rn_hi, rn_lo, staged_rows);
 }
 
 // Host: rows a tile must stage, the largest over every tile of the scene:
