@@ -30,6 +30,9 @@ sar_status fail(sar_status st, const char *fmt, ...) {
     vsnprintf(buf, sizeof(buf), fmt, ap);
     va_end(ap);
     g_last_error = buf;
+    // a reported error leaves the runtime's record: the next launch that asks for
+    // the last error (cudaGetLastError after <<<>>>) would take it for its own
+    if (st == SAR_ERR_CUDA) cudaGetLastError();
     return st;
 }
 
