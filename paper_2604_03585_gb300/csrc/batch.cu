@@ -183,9 +183,18 @@ static int64_t batch_inject_strip() {
     return v ? atoll(v) : -1;
 }
 
+// Test hook (host-side fault injection): batches created while
+// SAR_FAULT_INJECT_BATCH_SCRATCH=1 find no memory for the scratch of their
+// long range items, with 2 none for the tables beside the scratch.
+static int batch_inject_scratch() {
+    const char *v = getenv("SAR_FAULT_INJECT_BATCH_SCRATCH");
+    return v ? atoi(v) : 0;
+}
+
 // The one-launch batch: classes and their tables, the strip and item tables,
-// and a graph of one memset (the counters) and one kernel.
-static sar_status create_persistent(const sar_strip *strips, int32_t count, sar_batch b) {
+// and a graph of one memset (the counters) and one kernel.  The scratch of
+// long range items is taken only with may_park.
+static sar_status create_persistent(const sar_strip *strips, int32_t count, bool may_park, sar_batch b) {
     struct TClass {
         const SchedDesc *d;
         const void *spectrum;
@@ -248,9 +257,9 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, sar_
     };
     bool parks = false;
     for (int32_t i = 0; i < count; ++i) parks = parks || range_geometry(strips[i].n_range).parks;
-    if (parks) {
+    if (parks && may_park) {
         const size_t bytes = sizeof(float2) * (size_t)sar::batch_grid() * sar::kBatchScratch;
-        if (cudaMalloc(&b->work, bytes) == cudaSuccess) {
+        if (batch_inject_scratch() != 1 && cudaMalloc(&b->work, bytes) == cudaSuccess) {
             b->work_bytes = (int64_t)bytes;
         } else {
             cudaGetLastError();
@@ -323,8 +332,9 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, sar_
     const size_t off_ctr = reserve(sizeof(int) * ((size_t)count + sar::kBatchNumLists));
     const size_t off_status = reserve(sizeof(int));
     const size_t off_ix = reserve(sizeof(int32_t) * max_n);
-    if (cudaMalloc(&b->tables, tab) != cudaSuccess) {
+    if ((b->work && batch_inject_scratch() == 2) || cudaMalloc(&b->tables, tab) != cudaSuccess) {
         cudaGetLastError();
+        b->tables = nullptr;
         return sar::report_error(SAR_ERR_OUT_OF_MEMORY, "batch tables");
     }
     char *base = (char *)b->tables;
@@ -431,12 +441,23 @@ sar_status sar_batch_create(const sar_strip *strips, int32_t count, uint32_t fla
     cudaGetDevice(&b->device);
     b->strips = count;
     if (!multi) {
-        for (int32_t i = 0; i < count; ++i) b->samples += strips[i].n_az * strips[i].n_range;
-        const sar_status pst = create_persistent(strips, count, b);
+        sar_status pst = create_persistent(strips, count, true, b);
+        if (pst != SAR_OK && b->work) {
+            // the scratch only makes a batch faster: without it where the rest then finds no memory
+            const sar_batch again = new (std::nothrow) sar_batch_s;
+            if (again) {
+                again->device = b->device;
+                again->strips = count;
+                batch_free(b);
+                b = again;
+                pst = create_persistent(strips, count, false, b);
+            }
+        }
         if (pst != SAR_OK) {
             batch_free(b);
             return pst;
         }
+        for (int32_t i = 0; i < count; ++i) b->samples += strips[i].n_az * strips[i].n_range;
         *out = b;
         return SAR_OK;
     }

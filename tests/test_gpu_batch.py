@@ -176,6 +176,37 @@ def test_one_launch_mixed_lengths_equals_multi_kernel_graph(sar, shapes):
     one.destroy()
 
 
+@pytest.mark.parametrize("inject", ["1", "2"], ids=["no_scratch", "no_tables_beside_it"])
+def test_batch_without_memory_for_the_scratch(sar, monkeypatch, inject):
+    """Long range lines are parked in a scratch; where the device has no memory for it, or none for the
+    tables beside it, the batch is created without and gives the same images."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    c64 = lambda *s: torch.randn(s, dtype=torch.complex64, device="cuda", generator=gen)
+    strips = []
+    for r, a in [(8192, 16 * sms + 3), (16384, 12 * sms + 1), (8192, 5)]:     # a third above where sets begin
+        L = max(256, 1 << (a - 1).bit_length())
+        strips.append(dict(n_range=r, n_az=a, raw=c64(a, r), range_spectrum=c64(r), az_spectrum=c64(L),
+                           image=torch.empty((r, a), dtype=torch.complex64, device="cuda")))
+    images = []
+    for hook in (None, inject):
+        if hook:
+            monkeypatch.setenv("SAR_FAULT_INJECT_BATCH_SCRATCH", hook)
+        batch = sar.sar_batch_create(strips)
+        monkeypatch.delenv("SAR_FAULT_INJECT_BATCH_SCRATCH", raising=False)
+        info = sar.sar_batch_info(batch)
+        assert (info["work_bytes"] > 0) == (hook is None)
+        assert info["strips"] == 3 and info["samples"] == sum(st["raw"].numel() for st in strips)
+        for st in strips:
+            st["image"].fill_(float("nan"))
+        sar.sar_batch_run(batch)
+        sar.sar_batch_status(batch)
+        images.append([st["image"].clone() for st in strips])
+        batch.destroy()
+    for one, other in zip(*images):
+        assert torch.equal(one, other)
+
+
 def test_ragged_batch_wait_timeout_is_reported(sar):
     """A strip whose completion counter can never reach its target
     (host-side injection: one range line more expected than it has) makes the
