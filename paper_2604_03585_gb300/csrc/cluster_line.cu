@@ -35,6 +35,8 @@
 // memory in natural k2 order (stride C in the output line).
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "launch.cuh"
 #include "registry.h"
 
@@ -229,10 +231,15 @@ cluster_streamed_kernel(const float2* in, float2* out, int64_t ld, const float2*
 }
 
 // Stand-alone FFT of a line, natural-order output (unnormalised; the inverse
-// as conj(FFT(conj x))).  Output lines are dense lines of N.
-template <class SC, int C, bool INV>
-__global__ void __launch_bounds__(SC::T)
+// as conj(FFT(conj x))).  Output lines are dense lines of N.  M = 8192 in
+// clusters of four and eight runs its passes over the whole line: warp-local
+// they take 176 registers, which leaves one block per SM (608 lines of 65536:
+// 335 us against 493; 2000 lines 1.07 against 1.60 ms).  Warp-local and capped at
+// 128 it is 1 to 7 % slower than line-wide.
+template <class SC_, int C, bool INV>
+__global__ void __launch_bounds__(SC_::T)
 cluster_dft_kernel(const float2* in, float2* out, int64_t ld, int valid, const float2* tw) {
+    using SC = std::conditional_t<SC_::N == 8192 && C <= 8, LineWide<SC_>, SC_>;
     namespace cg = cooperative_groups;
     using G = ClusterGeom<SC, C>;
     extern __shared__ float2 smem_dyn[];

@@ -76,6 +76,13 @@ __device__ __forceinline__ int pass_group(int t, int s) {
         return t + SC::T * s;
 }
 
+// The schedule with every pass over the whole line, for kernels that the group
+// order of WARP_LOCAL makes slower.  Tables and results are the same.
+template <class SC>
+struct LineWide : SC {
+    static constexpr bool WARP_LOCAL = false;
+};
+
 // --- shared-memory exchange ----------------------------------------------
 template <class SC, int R, int S>
 __device__ __forceinline__ void smem_store(float2* sm, int t, const float2 (&v)[SC::E]) {

@@ -163,3 +163,22 @@ def test_long_lines_refused_where_unsupported(sar):
     with pytest.raises(sar.SarError) as e:
         sar.sar_plan_create(256, 262144, a, a)
     assert e.value.status == sar.SAR_ERR_UNSUPPORTED
+
+
+def test_transforms_of_long_lines_cost_alike(sar):
+    """Per sample, 65536 points cost what 32768 cost, within a few percent (blocks of both fill an SM
+    alike; a kernel that has lost its second block per SM takes 1.6 times as long)."""
+    per_sample = {}
+    for n in (32768, 65536):
+        x = torch.randn((1 << 25) // n, n, dtype=torch.complex64, device="cuda")
+        y = torch.empty_like(x)
+        times = []
+        for _ in range(12):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            sar.sar_fft_lines(n, x.shape[0], x, y)
+            end.record()
+            end.synchronize()
+            times.append(start.elapsed_time(end))
+        per_sample[n] = min(times)
+    assert per_sample[65536] < 1.3 * per_sample[32768], per_sample
