@@ -156,9 +156,13 @@ __device__ __forceinline__ void streamed_final_group(const float2* sm, const flo
     dft_reg<SC::R1, true>(x);
 }
 
-template <class SC, int LPB, bool ROLL>
+// Two forms keep the line-wide order (16384 lines of 4096): E = 16, which has no
+// registers to spare for the other (276.5 us against 288.6), and the cap of five
+// blocks per SM, where the other spills (256.5 against 261.9).
+template <class SC_, int LPB, bool ROLL>
 __device__ __forceinline__ void fused_streamed_body(const float2* in, float2* out, int64_t n_lines, int64_t ld,
                                                     const float2* filt, const float2* tw) {
+    using SC = std::conditional_t<(SC_::E == 16 && SC_::N == 4096) || SC_::MINB == 5, LineWide<SC_>, SC_>;
     extern __shared__ float2 smem_dyn[];
     grid_wait_predecessor();
     const int lib = threadIdx.x / SC::T;
