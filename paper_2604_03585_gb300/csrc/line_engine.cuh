@@ -44,6 +44,7 @@ struct Sched {
     // After pass 1 a line is R1 independent sub-lines of S1 consecutive
     // positions.  Where a warp's 32 E elements are whole sub-lines, the passes
     // between the forward and the inverse pass 1 stay inside the warp.
+    static constexpr bool STAGGER = true;   // staggered starts, where the line is long enough for them
     static constexpr bool WARP_LOCAL = P == 3 && T % 32 == 0 && (32 * E) % S1 == 0;
     static_assert(R1 * R2 * R3 == N, "radices must multiply to N");
     static_assert(E % R1 == 0 && E % R2 == 0 && E % R3 == 0, "each radix must divide E");
@@ -83,6 +84,11 @@ __device__ __forceinline__ int pass_group(int t, int s) {
 template <class SC>
 struct LineWide : SC {
     static constexpr bool WARP_LOCAL = false;
+};
+// The schedule without staggered starts (below), for kernels that lose with them.
+template <class SC>
+struct Unstaggered : SC {
+    static constexpr bool STAGGER = false;
 };
 
 // --- shared-memory exchange ----------------------------------------------
@@ -222,7 +228,7 @@ __device__ __forceinline__ void sub_sync(int line_in_block) {
 // lines per block; the lines of a block synchronise on ids 0 ... 8.
 template <class SC, int LPB>
 struct Stagger {
-    static constexpr bool ON = SC::WARP_LOCAL && SC::T >= 256 && LPB <= 2;
+    static constexpr bool ON = SC::STAGGER && SC::WARP_LOCAL && SC::T >= 256 && LPB <= 2;
     static constexpr int GROUP = ON ? SC::T / 4 : SC::T;
 };
 template <class SC, int LPB>
