@@ -229,34 +229,54 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, bool
         cudaGetLastError();
         return sar::report_error(SAR_ERR_CUDA, "the batch kernel does not fit the device");
     }
-    // how the range items of each length run.  Long lines are stored in sets of
-    // four, all but the last parked in the scratch (none if there is no memory
-    // for it: then an item is the lines its worker holds at once).  A few waves
-    // of such sets leave workers idle at the end: there the whole block takes
-    // as many lines as it holds and parks none.  One strip, us against us with
-    // sets: 4096 x 400 37 / 90, 4096 x 5000 466 / 526 (limit: four sets for
-    // each worker of 128 threads); 8192 x 300 53 / 108, x 1570 275 / 318, x 2400
-    // 486 / 427 (three per block); 16384 x 300 110 / 137, x 700 237 / 286, x
-    // 1500 580 / 543 (two per block)
+    // How the range items of each length run.  Up to 1024 samples the workers'
+    // own lines fill a set.  Longer lines go to the whole block, as many as it
+    // holds and none parked, or to workers of a quarter or half of it in sets of
+    // four, all but the last parked in the scratch (without memory for it an
+    // item is the lines that its worker holds).  Sets keep the lines of an SM
+    // out of phase, but a few waves of them leave workers idle at the end.  us
+    // whole / in sets, strips of azimuth lines x range samples:
+    // 2048 and 4096, together: sets from four for every worker.  4096: 1 strip of
+    //   4096 lines (1024 sets) 256 / 296, 2 of 4096 (2048) 494 / 497, 10 of 1000
+    //   (2500) 498 / 487, 3 of 4096 758 / 723, 12 of 4096 2882 / 2717.  2048: 1 of
+    //   4096 129 / 139, 2 of 4096 230 / 237, beyond that within 4 % either way (5 of
+    //   2000 290 / 300, 3 of 4096 350 / 346, 12 of 4096 1310 / 1327); beside 4096
+    //   and longer it gains (16 strips of 1024 ... 16384: 2776 / 2747).  Strips of
+    //   more than 4096 lines, whose azimuth items wait in another list, stay whole
+    //   and do not count: 4096 x 12000 lines 914 / 957, 3 of 8000 1518 / 1530, 2048
+    //   x 12000 438 / 454.
+    // 8192: sets from three per block.  1 of 1500 (375) 250 / 303, 1 of 2400 (600)
+    //   431 / 427, 4 of 1500 962 / 879; in between one strip loses (1 of 2100, 525:
+    //   401 / 409) and strips beside others gain (516 of 8192 among 9 strips of 2048
+    //   ... 16384: 1483 / 1457).
+    // 16384: sets from two per block.  1 of 900 (225) 280 / 297, 1 of 1500 (375)
+    //   564 / 539, 1 of 4096 1441 / 1200; shorter strips gain earlier (3 of 300
+    //   280 / 255).
     const int64_t blocks = sar::batch_grid(), workers = blocks * (sar::kBatchThreads / 128);
     int64_t sets_short = 0, sets_8192 = 0, sets_16384 = 0, sets_tiny = 0;
     for (int32_t i = 0; i < count; ++i) {
         const int64_t sets = (strips[i].n_az + sar::kLongLines - 1) / sar::kLongLines;
         if (strips[i].n_range == 16384) sets_16384 += sets;
         else if (strips[i].n_range == 8192) sets_8192 += sets;
-        else if (strips[i].n_range >= 2048) sets_short += sets;
+        else if (strips[i].n_range >= 2048 && strips[i].n_az <= 4096) sets_short += sets;
         else if (strips[i].n_range <= 512) sets_tiny += (strips[i].n_az + 7) / 8;
     }
-    auto few = [&](int64_t n) {
-        return n == 16384 ? sets_16384 < 2 * blocks : n == 8192 ? sets_8192 < 3 * blocks : sets_short < 4 * workers;
+    auto whole_block = [&](const sar_strip &s) {
+        switch (s.n_range) {
+            case 2048:
+            case 4096: return s.n_az > 4096 || sets_short < 4 * workers;
+            case 8192: return sets_8192 < 3 * blocks;
+            case 16384: return sets_16384 < 2 * blocks;
+            default: return false;
+        }
     };
-    auto range_geometry = [&](int64_t n) {
-        sar::BatchGeom g = sar::batch_geometry((int)n, few(n));
-        if (n >= 8192 && few(n)) g.parks = false, g.set = g.lines;
+    auto range_geometry = [&](const sar_strip &s) {
+        sar::BatchGeom g = sar::batch_geometry((int)s.n_range, whole_block(s));
+        if (s.n_range >= 8192 && whole_block(s)) g.parks = false, g.set = g.lines;
         return g;
     };
     bool parks = false;
-    for (int32_t i = 0; i < count; ++i) parks = parks || range_geometry(strips[i].n_range).parks;
+    for (int32_t i = 0; i < count; ++i) parks = parks || range_geometry(strips[i]).parks;
     if (parks && may_park) {
         const size_t bytes = sizeof(float2) * (size_t)sar::batch_grid() * sar::kBatchScratch;
         if (batch_inject_scratch() != 1 && cudaMalloc(&b->work, bytes) == cudaSuccess) {
@@ -294,7 +314,7 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, bool
         }
         for (int32_t i : order) {
             const sar::BatchGeom g =
-                range ? range_geometry(strips[i].n_range) : sar::batch_geometry((int)L[i]);
+                range ? range_geometry(strips[i]) : sar::batch_geometry((int)L[i]);
             if (g.threads != threads) continue;
             const int64_t lines = range ? strips[i].n_az : strips[i].n_range, n = range ? strips[i].n_range : L[i];
             const int unit = range && (b->work || !g.parks) ? g.set : g.lines;

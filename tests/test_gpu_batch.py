@@ -139,17 +139,32 @@ def test_one_launch_equals_multi_kernel_graph(sar):
     multi.destroy()
 
 
-@pytest.mark.parametrize("shapes", [
-    # azimuth lengths 512 ... 4096 side by side in the workers of a block, several lines per worker item,
-    # range items of 8192 and 16384 samples in two and four rounds with a remainder
-    [(4096, 4101), (4096, 3001), (8192, 1830), (16384, 1222), (2048, 1026), (4096, 2049)],
+def _mixed_workers(sms):
+    # azimuth lengths 512 ... 4096 side by side in the workers of a block, several lines per worker item, range
+    # items of 4096, 8192 and 16384 samples in sets of parked lines (a third above the least number) with a remainder
+    return [(4096, 4001)] * -(-75 * sms // 4001) + [(8192, 20 * sms + 2), (16384, 12 * sms + 2), (2048, 1026), (4096, 2049)]
+
+
+def _whole_block(sms):
+    # range lines of 2048 and 4096 samples that never park, however many: strips of more than 4096 lines
+    return [(4096, 64 * sms + 1), (2048, 80 * sms + 3), (4096, 5)]
+
+
+def _long_azimuth(sms):
     # azimuth lines of the whole block (8192, 16384) beside short ones, few items
-    [(256, 4097), (512, 9000), (8192, 3), (16384, 5), (16384, 1), (1024, 257)],
+    return [(256, 4097), (512, 9000), (8192, 3), (16384, 5), (16384, 1), (1024, 257)]
+
+
+def _many_short(sms):
     # several sets of short range lines per item, with a remainder
-    [(256, 16384), (512, 12001), (256, 3001)],
-], ids=["mixed_workers", "long_azimuth", "many_short"])
-def test_one_launch_mixed_lengths_equals_multi_kernel_graph(sar, shapes):
+    return [(256, 16384), (512, 12001), (256, 3001)]
+
+
+@pytest.mark.parametrize("shapes,parks", [(_mixed_workers, True), (_whole_block, False), (_long_azimuth, False),
+                                          (_many_short, False)], ids=lambda p: getattr(p, "__name__", None))
+def test_one_launch_mixed_lengths_equals_multi_kernel_graph(sar, shapes, parks):
     """Same engines, the corner turn a copy: bit-identical images, twice in a row."""
+    shapes = shapes(torch.cuda.get_device_properties(0).multi_processor_count)
     gen = torch.Generator(device="cuda").manual_seed(11)
     c64 = lambda *s: torch.randn(s, dtype=torch.complex64, device="cuda", generator=gen)
     hr = {r: c64(r) for r, _ in shapes}
@@ -166,6 +181,7 @@ def test_one_launch_mixed_lengths_equals_multi_kernel_graph(sar, shapes):
     want = [st["image"].clone() for st in strips]
     multi.destroy()
     one = sar.sar_batch_create(strips)
+    assert (sar.sar_batch_info(one)["work_bytes"] > 0) == parks
     for _ in range(2):
         for st in strips:
             st["image"].fill_(float("nan"))
@@ -184,7 +200,7 @@ def test_batch_without_memory_for_the_scratch(sar, monkeypatch, inject):
     gen = torch.Generator(device="cuda").manual_seed(5)
     c64 = lambda *s: torch.randn(s, dtype=torch.complex64, device="cuda", generator=gen)
     strips = []
-    for r, a in [(8192, 16 * sms + 3), (16384, 12 * sms + 1), (8192, 5)]:     # a third above where sets begin
+    for r, a in [(8192, 20 * sms + 3), (16384, 12 * sms + 1), (8192, 5)]:     # well above where sets begin
         L = max(256, 1 << (a - 1).bit_length())
         strips.append(dict(n_range=r, n_az=a, raw=c64(a, r), range_spectrum=c64(r), az_spectrum=c64(L),
                            image=torch.empty((r, a), dtype=torch.complex64, device="cuda")))
