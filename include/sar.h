@@ -356,17 +356,21 @@ typedef struct {
  * filter: range classes by (n_range, range spectrum), azimuth classes by (L,
  * azimuth spectrum)), build each class's filter and twiddle tables, and
  * capture the whole batch into one CUDA graph.
- * flags 0: the graph is one memset and ONE persistent kernel.  Each resident
- * block (one per SM) takes work items: first range items (at least four
- * azimuth rows of a strip, compressed along range and written straight into
- * the corner-turned image, Sec. IV-A steps 1-2), then each quarter of the
- * block azimuth items (range bins, compressed along azimuth in place, Sec.
- * IV-A step 4; above 4096 samples the whole block).
+ * flags 0: the graph is one memset and ONE persistent kernel.  One block per
+ * SM is resident, as one, two or four workers by the length of the lines, and
+ * takes work items: range items (azimuth rows of a strip, compressed along
+ * range and written straight into the corner-turned image, Sec. IV-A steps
+ * 1-2), then azimuth items (range bins, compressed along azimuth in place, Sec.
+ * IV-A step 4).  Azimuth lines of up to 4096 samples run on quarters of the
+ * block, 8192 on halves, 16384 on the whole block.  A range item is at least
+ * four rows, but two of 8192 or one of 16384 samples where there are few of
+ * them, and the one or two that a worker holds where there is no scratch.
  * A strip's azimuth items wait on a device counter of its finished range
  * lines; that wait is bounded (about a second of SM clock, SAR_WAIT_CYCLES),
  * and a run whose wait ran out is reported by sar_batch_status.  No work
- * buffer, but for strips of 8192 or 16384 range samples a scratch of up to
- * 384 KiB per SM (without memory for it those strips run slower).
+ * buffer; a batch of many range lines of 2048 samples or more owns a scratch of
+ * 384 KiB per SM (work_bytes), and is created without it, and runs slower,
+ * where the device has no memory for it.
  * flags SAR_BATCH_MULTI_KERNEL or SAR_BATCH_EXACT_AZIMUTH: see below (one
  * launch per class, a batched corner turn, a work buffer of 8 bytes per raw
  * sample).

@@ -5,11 +5,11 @@
 // count); its azimuth lines are transformed at L = max(256, next power of
 // two >= n_az), zero-padded, and the image keeps its n_az columns.
 //
-// Default: one persistent kernel (batch_persistent.cu) walks two lists of work
-// items -- range items (k azimuth rows of a strip, compressed along range and
-// written corner-turned into the image) and azimuth items (k range bins,
-// compressed in place) -- with per-strip completion counters between a
-// strip's range and azimuth items.  The graph is one memset of the counters
+// Default: one persistent kernel (batch_persistent.cu) walks five lists of work
+// items, by the threads of a worker -- range items (azimuth rows of a strip,
+// compressed along range and written corner-turned into the image), then azimuth
+// items (range bins, compressed in place) -- with per-strip completion counters
+// between a strip's range and azimuth items.  The graph is one memset of the counters
 // and that one kernel.  Filters and twiddles are built per class: range
 // classes by (n_range, range spectrum), azimuth classes by (L, azimuth
 // spectrum), on the kernel's engine geometry of each length.
@@ -291,9 +291,9 @@ static sar_status create_persistent(const sar_strip *strips, int32_t count, bool
     // whose 32-byte runs share the image rows' L2 lines, are stored at about
     // the same time (1024 x 3651 strips: 228 us per 2^24 samples against 271
     // with four sets per item), or up to 8192 samples of lines up to 512, where
-    // taking the item would cost more (256 x 4096: 176 against 204); an azimuth item of 128 threads is up to four rounds of its worker's
-    // lines where that leaves every worker several (256 x 4096: 176 against
-    // 208 with one)
+    // taking the item would cost more (256 x 4096: 176 against 204); an azimuth
+    // item of 128 threads is up to four rounds of its worker's lines where that
+    // leaves every worker several (256 x 4096: 176 against 208 with one)
     std::vector<int32_t> order(count);
     for (int32_t i = 0; i < count; ++i) order[i] = i;
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {

@@ -105,7 +105,8 @@ constexpr int kSmem = (kSmemElems + 4 * kWorkElems) * (int)sizeof(float2);
 // item routines, which are calls, find it by this name and not through a
 // pointer argument, and say which pointers are global ones: behind a generic
 // pointer every exchange and table access is a generic load, which waits like
-// a global one (azimuth lines of 4096: @@GEN@@).
+// a global one (16 strips of 256 lines of 4096: 193 us against 231, 3 of 4096 x
+// 4096 715 against 858).
 extern __shared__ __align__(16) float2 batch_smem[];
 __device__ __forceinline__ BWork& work_of(int w) {
     return reinterpret_cast<BWork*>(batch_smem + kSmemElems)[w];

@@ -6,12 +6,21 @@
 
 namespace sar {
 
-// Up to this many threads in all, about two waves of the GPU, the time from
-// one kernel's end to the next one's first instruction counts: it is then
-// launched while its predecessor still runs and waits for it in the kernel
-// (sar_common.cuh: grid_wait_predecessor, with which every kernel launched here
-// begins).
-// Above, blocks that wait would only keep SMs from other streams' kernels.
+// Up to this many threads in all, the time from one kernel's end to the next
+// one's first instruction counts: it is then launched while its predecessor still
+// runs and waits for it in the kernel (sar_common.cuh: grid_wait_predecessor).
+// Every kernel launched here waits before it touches the caller's data or anything
+// that a kernel of the library writes.  Before it, the kernels for few short lines
+// read the plan's twiddles and filter: whoever hands tables to a launch has
+// waited on the host until they were complete.
+// The limit is in threads: two waves of the GB300's 152 SMs of kernels that fill
+// them, and up to eight of the three-pass engines, which hold 512 threads per SM.
+// It saves two to five us a scene: 1024 x 1024 18.6 -> 15.3, 2048 x 4096 84.5 ->
+// 80.0, 4096 x 4096 158.0 -> 153.3.  Larger passes would save as much, below 2 %
+// of theirs (8192 x 4096: 320 -> 316), and are launched ordinarily: blocks that
+// wait hold slots that another stream's kernels could use.  (On four streams and in
+// serving neither side of the limit showed a difference: 8.4 us a scene of 1024
+// x 1024 either way, 8.9 without.)
 constexpr int64_t kBehindThreads = 2 * 152 * 2048;
 // Clusters are not where they take part of the GPU's slots: placed while the
 // predecessor's last blocks still hold some, they crowd on the others (256
