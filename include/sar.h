@@ -387,7 +387,7 @@ typedef struct {
  * (zero-padded) semantics: one fused launch per class walking a segment
  * table, one batched corner turn, a work buffer of 8 bytes per raw sample.
  * On GB300 it runs large batches faster than the one-launch kernel (64 strips
- * of 948 M samples in all: 11.8 against 16.8 ms), whose blocks are sized for
+ * of 948 M samples in all: 11.7 against 16.4 ms), whose blocks are sized for
  * 16384-sample lines, one per SM, while the per-class kernels run four or five
  * blocks per SM. */
 #define SAR_BATCH_MULTI_KERNEL 2u

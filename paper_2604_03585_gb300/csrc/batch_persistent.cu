@@ -13,7 +13,7 @@
 // and one loads while another computes, as in the one-length kernels with
 // four blocks per SM.  Bound by latency (one block, sixteen warps per SM:
 // issue 38 %, L1 55 %).  16 strips of 1024 ... 16384 x 337 ... 4054 samples
-// (148 M): 2.73 ms, against 3.07 with items of the whole block throughout and
+// (148 M): 2.71 ms, against 3.07 with items of the whole block throughout and
 // every exchange and table access through generic pointers; 1024 x 256 strips
 // 150 us per 2^24 samples against 283, 4096 x 256 177 against 255, 16384 x 256
 // 234 against 327.

@@ -92,7 +92,7 @@ __device__ __forceinline__ float2 at(float2 v) {
 // (rows n0 + min shift - 7 ... n0 + 127 + max shift + 8, zero outside the
 // scene); the host sizes that span from the geometry, and a block whose span
 // does not fit reads global memory directly.
-// Bound by ALU issue: 178 thread instructions per output (223 with the weights
+// Bound by ALU issue: 177 thread instructions per output (223 with the weights
 // from reciprocals and sines; the floor of the 4096 x 4096 scene's 268 MB is 40
 // us, of its instructions 74).  102.8 us at 4096 x 4096, from 122.5: polynomial
 // weights for two outputs at once 105.0 (one at a time 123.5, four 108.8, with
